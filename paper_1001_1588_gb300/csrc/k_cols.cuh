@@ -129,6 +129,7 @@ __global__ void __launch_bounds__((NY / V > 256) ? 512 : 256, 1) col_stats_kerne
       phase ^= 1;
       float2 v[V];
       read_line<NY, V>(v, stage, t, part);
+      stage_reads_done();
       __syncthreads();                                   // stage consumed
       if (threadIdx.x == 0) {
         if (l + 1 < lines_per_col) issue(cb, l + 1);
@@ -431,6 +432,7 @@ __global__ void __launch_bounds__((NY / V > 256) ? 512 : 256, 1) col_update_kern
           }
         }
       }
+      stage_reads_done();   // the gain stage, and the innovation stage read before it
       __syncthreads();   // gain stage consumed
       if (threadIdx.x == 0) {
         if (j + 1 < p.M) issue_g(base, j + 1);

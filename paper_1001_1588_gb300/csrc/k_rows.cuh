@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(512, 1) row_fwd_kernel(const RowFwdParams p) {
           v[m] = make_float2(sv[m].x - a.x, sv[m].y - a.y);
         }
       }
+      stage_reads_done();
       __syncthreads();   // stage consumed
       if (threadIdx.x == 0) {
         if (r + 1 < rounds) issue(q, r + 1);
@@ -286,6 +287,7 @@ __global__ void __launch_bounds__(512, 1) row_anom_kernel(const RowFwdParams p) 
             const float2 a = load2<ST>(st_row, 2 * (size_t)(t + T * m));
             v[m] = make_float2(a.x - sv[m].x, a.y - sv[m].y);
           }
+          stage_reads_done();
           __syncthreads();   // stage consumed
           if (threadIdx.x == 0) {
             const int s = (k - 1) * rounds + r + 1;
@@ -413,6 +415,7 @@ __global__ void __launch_bounds__(512, 1) row_inv_kernel(const __grid_constant__
       line[pidx(c)] = make_float2(A.x - Bw.y, A.y + Bw.x);
       if (c != L - c) line[pidx(L - c)] = make_float2(A.x + Bw.y, Bw.x - A.y);
     }
+    stage_reads_done();
     __syncthreads();   // tile consumed, rows staged
     if (threadIdx.x == 0 && q + gridDim.x < Q) issue_tile(q + gridDim.x);
     float2* line = lines + (size_t)g * pitch;
@@ -430,6 +433,7 @@ __global__ void __launch_bounds__(512, 1) row_inv_kernel(const __grid_constant__
     float2 a[V];
 #pragma unroll
     for (int m = 0; m < V; ++m) a[m] = load2<ST>(st_row, 2 * (size_t)(t + T * m));
+    stage_reads_done();
     __syncthreads();   // stage consumed
     if (threadIdx.x == 0 && q + gridDim.x < Q) issue_rows(q + gridDim.x);
     char* urow = ens + (f * G + (size_t)(y0 + g) * nx) * es;

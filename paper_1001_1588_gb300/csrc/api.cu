@@ -15,6 +15,8 @@
 // wide column schedule), steps 3 and 6 are one launch after step 5:
 //   5. row_fwd innov, 3+6. col_fused (columns of F, chat, gains, gain x innovation, inverse
 //   columns -> S), 7. row_inv.
+// Small grids and ensembles take the passes of k_split.cuh instead (split_rule): 2 and 5 in one launch,
+// 3, 4 and 6 in one launch that reads rhat or the caller's spectrum as they are, 7.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -295,6 +297,59 @@ static fftenkf_status get_workspace(fftenkf_plan p, void* ws, char** out) {
   return FFTENKF_OK;
 }
 
+// Which passes of a call run split into independent CTAs (k_split.cuh): bit 0 the forward rows, bit 1
+// the columns, bit 2 the inverse rows.  Measured on a 152-SM GB300 (us, pipelined passes -> split):
+//   rows: 64^2 N=5 27 -> 8, 512^2 N=20 71 -> 34, 1536x768 N=25 3 blocks 382 -> 259, 2048^2 N=20 4 blocks
+//     1088 -> 1025; rows of 4096 points only where the pipelined pass has fewer tiles of 8 rows than half
+//     the SMs (256x4096 N=4 66 -> 39, but 512x4096 N=20 4 blocks 597 -> 841)
+//   columns: up to 768 points always (512^2 N=5 3 blocks 101 -> 30, 512x4096 N=20 4 blocks 683 -> 598);
+//     above, with one observed and no other block (1024^2 N=20 163 -> 100, 2048^2 N=10 352 -> 213), with all
+//     blocks observed at 1024 (186 -> 187, two launches fewer), where the fused pass does not apply for the
+//     observed blocks (1024x2048 N=15, 3 of 4 observed 851 -> 672), and where the fused pass would leave
+//     more than half its column groups idle (1024x512 N=8 167 -> 104, but 1024^2 N=20 192 -> 218)
+//   inverse rows: up to 2^23 points of the ensemble and 2048-point rows (1024^2 N=5 25 -> 21, but N=20 65 -> 72)
+enum SplitBits { kSplitRows = 1, kSplitCols = 2, kSplitInv = 4 };
+static int split_rule(fftenkf_plan p) {
+  for (int a = 0; a < kPassCount; ++a)
+    if (p->sched[a] != 0) return 0;   // a schedule was chosen: the passes it names
+  int bits = 0;
+  if (p->expire_first_wait == 0 && split_rows_supported(p->L) && (p->L <= 1024 || 2 * p->M * (p->ny / 8) <= sm_count()))
+    bits |= kSplitRows;
+  if (!p->coupled && split_cols_supported(p->ny, p->n_obs, p->M)) {
+    const bool all = p->n_un == 0;
+    if (p->ny <= 768 || (p->ny == 1024 && all) || p->M == 1 || (p->ny == 1024 && p->n_obs > 2) ||
+        (p->use_fused() && 2 * (p->L + 1) <= col_fused_groups(p->ny, 0)))
+      bits |= kSplitCols;
+  }
+  if (p->L <= 1024 && (long long)p->M * p->N * p->ny * p->nx <= (1LL << 23)) bits |= kSplitInv;
+  return bits;
+}
+
+static SplitParams split_params(fftenkf_plan p, char* ws, const void* ens, const float* data, const void* pert,
+                                const double* rhat) {
+  SplitParams q;
+  memset(&q, 0, sizeof(q));
+  q.ny = p->ny; q.nx = p->nx; q.L = p->L; q.M = p->M; q.n_obs = p->n_obs; q.n_un = p->n_un; q.storage = p->storage;
+  for (int i = 0; i < p->n_obs; ++i) q.obs[i] = p->obs[i];
+  for (int r = 0; r < p->M; ++r) q.role_block[r] = (r < p->n_obs) ? p->obs[r] : p->un[r - p->n_obs];
+  q.one.N = p->N;
+  q.one.inv_sqrt_N = (float)(1.0 / std::sqrt((double)p->N));
+  q.one.scale = (float)(1.0 / ((double)(p->N - 1) * (double)p->ny * (double)p->nx));
+  q.one.ens = const_cast<void*>(ens);   // written by the inverse rows only
+  q.one.data = data;
+  q.one.pert = pert;
+  q.one.rhat = rhat;
+  q.one.A = reinterpret_cast<float2*>(ws + p->off_A);
+  q.one.W = reinterpret_cast<float2*>(ws + p->off_W);
+  q.twL = p->twL(split_row_V(p->L) == plan_V(p->L, 0) ? 0 : 1);
+  q.twX = p->twX();
+  q.twY = p->twY(split_col_sel(p->ny, p->n_un > 0));
+  q.inv_G = (float)(1.0 / ((double)p->ny * (double)p->nx));
+  q.sqrt_G = (float)std::sqrt((double)p->ny * (double)p->nx);
+  q.status = p->d_status;
+  return q;
+}
+
 static ColFusedParams fused_params(fftenkf_plan p, char* ws) {
   ColFusedParams f;
   memset(&f, 0, sizeof(f));
@@ -327,12 +382,49 @@ static cudaError_t run_anomaly_rows(fftenkf_plan p, const void* ens, char* ws, c
   return e;
 }
 
-// steps 2-3: anomaly row spectra, column statistics -> chat_t
+// innovation row spectra -> W
+static cudaError_t run_innovation_rows(fftenkf_plan p, const void* ens, const float* data, const void* pert, int mode,
+                                       char* ws, cudaStream_t s) {
+  RowFwdParams rp;
+  memset(&rp, 0, sizeof(rp));
+  rp.ny = p->ny; rp.nx = p->nx; rp.L = p->L; rp.M = p->M; rp.N = p->N;
+  rp.n_obs = p->n_obs; rp.mode = mode; rp.storage = p->storage;
+  for (int i = 0; i < p->n_obs; ++i) rp.obs[i] = p->obs[i];
+  rp.ens = ens; rp.data = data; rp.pert = pert;
+  rp.out = reinterpret_cast<float2*>(ws + p->off_W);
+  rp.vsel = p->sched[kPassRowInnov];
+  rp.twL = p->twL(rp.vsel & 1); rp.twX = p->twX(); rp.status = p->d_status;
+  prof_begin(p, kPassRowInnov, s);
+  cudaError_t e = launch_row_fwd(rp, p->N * p->n_obs, s);
+  prof_end(p, kPassRowInnov, s);
+  return e;
+}
+
+// The forward rows of an analysis or estimate: the anomalies (step 2) and the innovations (step 5;
+// 0, kInnovation or kInnovationDrawn).  Split, both are one launch, timed as the anomaly rows.
+static cudaError_t run_rows(fftenkf_plan p, const SplitParams& q, bool anomalies, int innovations, int split, char* ws,
+                            cudaStream_t s) {
+  if (split & kSplitRows) {
+    SplitParams r = q;
+    r.anomalies = anomalies ? 1 : 0;
+    r.innovations = innovations;
+    const int pass = anomalies ? kPassRowAnom : kPassRowInnov;
+    prof_begin(p, pass, s);
+    cudaError_t e = launch_row_split(r, s);
+    prof_end(p, pass, s);
+    return e;
+  }
+  cudaError_t e = cudaSuccess;
+  if (anomalies) e = run_anomaly_rows(p, q.one.ens, ws, s);
+  if (e == cudaSuccess && innovations) e = run_innovation_rows(p, q.one.ens, q.one.data, q.one.pert, innovations, ws, s);
+  return e;
+}
+
+// steps 3: column statistics of the anomaly row spectra -> chat_t
 // with rhat_t != null the column pass also forms the gains (analysis) and skips chat_t
-static cudaError_t run_statistics(fftenkf_plan p, const void* ens, char* ws, cudaStream_t s, const double* rhat_t,
+static cudaError_t run_statistics(fftenkf_plan p, char* ws, cudaStream_t s, const double* rhat_t,
                                   cudaEvent_t wait_before_stats = nullptr) {
-  cudaError_t e = run_anomaly_rows(p, ens, ws, s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   ColStatsParams cp;
   memset(&cp, 0, sizeof(cp));
   cp.ny = p->ny; cp.L = p->L; cp.M = p->M; cp.N = p->N; cp.n_obs = p->n_obs; cp.n_un = p->n_un;
@@ -377,7 +469,17 @@ extern "C" fftenkf_status fftenkf_estimate_spectrum(fftenkf_plan p, const void* 
   fftenkf_status st = get_workspace(p, workspace, &ws);
   if (st != FFTENKF_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = run_statistics(p, ensemble, ws, s, nullptr);
+  const int split = split_rule(p);
+  SplitParams q = split_params(p, ws, ensemble, nullptr, nullptr, nullptr);
+  cudaError_t e = run_rows(p, q, true, 0, split, ws, s);
+  if (split & kSplitCols) {
+    q.chat = reinterpret_cast<float*>(ws + p->off_chat);
+    prof_begin(p, kPassFused, s);
+    if (e == cudaSuccess) e = launch_col_split(q, s);
+    prof_end(p, kPassFused, s);
+  } else if (e == cudaSuccess) {
+    e = run_statistics(p, ws, s, nullptr);
+  }
   prof_begin(p, kPassChatOut, s);
   if (e == cudaSuccess)
     e = launch_chat_out(reinterpret_cast<float*>(ws + p->off_chat), spectrum_out, p->ny, p->L,
@@ -385,6 +487,100 @@ extern "C" fftenkf_status fftenkf_estimate_spectrum(fftenkf_plan p, const void* 
   prof_end(p, kPassChatOut, s);
   if (e != cudaSuccess) return cuda_fail(e, "estimate_spectrum");
   return FFTENKF_OK;
+}
+
+// Steps 2-6 with the pipelined column passes: forward rows, statistics, gains and update -> increment row spectra
+static cudaError_t run_columns(fftenkf_plan p, const SplitParams& q, const double* spectrum, bool drawn,
+                               unsigned long long seed, int split, char* ws, cudaStream_t s) {
+  const double* rhat = q.one.rhat;
+  const int innovations = drawn ? kInnovationDrawn : kInnovation;
+  const bool all_rows = (split & kSplitRows) != 0;   // anomalies and innovations in one launch
+  // auxiliary stream: rhat transposed for the gains (estimated spectrum) or the gain pass
+  // (caller spectrum), overlapping the passes on the caller's stream
+  cudaError_t e = cudaEventRecord(p->ev_fork, s);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(p->aux, p->ev_fork, 0);
+  GainParams gp;
+  memset(&gp, 0, sizeof(gp));
+  gp.ny = p->ny; gp.L = p->L; gp.n_obs = p->n_obs; gp.n_un = p->n_un;
+  gp.spec = spectrum;
+  gp.rhat = rhat;
+  gp.goo = reinterpret_cast<float*>(ws + p->off_goo);
+  gp.gjo = reinterpret_cast<float2*>(ws + p->off_gjo);
+  gp.scale = q.inv_G;
+  gp.status = p->d_status;
+  double* rhat_t = reinterpret_cast<double*>(ws + p->off_rhat_t);
+  const bool fused = !spectrum && p->use_fused();
+  float* amp_t = reinterpret_cast<float*>(ws + p->off_amp);
+  if (!spectrum || drawn) {   // drawn: the perturbations scale by sqrt(rhat) in the column layout
+    // the fused pass draws perturbations with the FP32 amplitudes sqrt(ny nx rhat) of the same pass
+    prof_begin(p, kPassRhatT, p->aux);
+    if (e == cudaSuccess)
+      e = launch_rhat_transpose(rhat, rhat_t, p->n_obs, p->ny, p->L, p->aux, (fused && drawn) ? amp_t : nullptr, q.sqrt_G);
+    prof_end(p, kPassRhatT, p->aux);
+  }
+  if (spectrum) {
+    prof_begin(p, kPassGain, p->aux);
+    if (e == cudaSuccess) e = launch_gain(gp, p->aux);
+    prof_end(p, kPassGain, p->aux);
+  }
+  if (e == cudaSuccess) e = cudaEventRecord(p->ev_join, p->aux);
+  if (e == cudaSuccess) e = run_rows(p, q, !spectrum, (all_rows || spectrum || fused) ? innovations : 0, split, ws, s);
+  if (fused) {
+    ColFusedParams f = fused_params(p, ws);
+    f.W = q.one.W;
+    f.rhat_t = rhat_t;
+    f.drawn = drawn ? 1 : 0;
+    f.seed = seed;
+    f.amp_t = amp_t;
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
+    prof_begin(p, kPassFused, s);
+    if (e == cudaSuccess) e = launch_col_fused(f, s);
+    prof_end(p, kPassFused, s);
+    return e;
+  }
+  if (spectrum) {
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
+  } else if (p->coupled) {
+    // tables of the column statistics, then the coupled gains (FP64 bracket inverse per wavenumber)
+    if (e == cudaSuccess) e = run_statistics(p, ws, s, nullptr);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
+    CoupledGainParams cg;
+    memset(&cg, 0, sizeof(cg));
+    cg.ny = p->ny; cg.L = p->L; cg.n_obs = p->n_obs; cg.n_un = p->n_un; cg.n_pair = p->n_pair;
+    cg.chat_t = reinterpret_cast<const float*>(ws + p->off_chat);
+    cg.rhat_t = rhat_t;
+    cg.gall = gp.gjo;
+    cg.inv_G = q.inv_G;
+    cg.status = p->d_status;
+    prof_begin(p, kPassGain, s);
+    if (e == cudaSuccess) e = launch_coupled_gain(cg, s);
+    prof_end(p, kPassGain, s);
+  } else {
+    // the statistics pass forms the gains and waits for rhat
+    if (e == cudaSuccess) e = run_statistics(p, ws, s, rhat_t, p->ev_join);
+  }
+  if (e == cudaSuccess && !spectrum && !all_rows) e = run_rows(p, q, false, innovations, split, ws, s);
+  ColUpdParams up;
+  memset(&up, 0, sizeof(up));
+  up.ny = p->ny; up.L = p->L; up.M = p->M; up.N = p->N; up.n_obs = p->n_obs; up.n_un = p->n_un;
+  for (int j = 0; j < p->M; ++j) {
+    up.obs_of_block[j] = p->obs_of_block[j];
+    up.un_of_block[j] = p->un_of_block[j];
+  }
+  up.W = q.one.W; up.goo = gp.goo; up.gjo = gp.gjo;
+  up.coupled = p->coupled ? 1 : 0;
+  up.gall = gp.gjo;
+  up.drawn = drawn ? 1 : 0;
+  up.seed = seed;
+  up.rhat_t = rhat_t;
+  up.sqrt_G = q.sqrt_G;
+  up.S = q.one.A;
+  up.vsel = p->sched[kPassUpdate];
+  up.twY = p->twY(up.vsel); up.status = p->d_status;
+  prof_begin(p, kPassUpdate, s);
+  if (e == cudaSuccess) e = launch_col_update(up, s);
+  prof_end(p, kPassUpdate, s);
+  return e;
 }
 
 // the analysis with given perturbations, or (drawn) with perturbations drawn in frequency space
@@ -404,129 +600,46 @@ static fftenkf_status analyze_impl(fftenkf_plan p, void* ensemble, const float* 
   fftenkf_status st = get_workspace(p, workspace, &ws);
   if (st != FFTENKF_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const int split = split_rule(p);
+  SplitParams q = split_params(p, ws, ensemble, data, perturbations, rhat);
+  const int innovations = drawn ? kInnovationDrawn : kInnovation;
   cudaError_t e = cudaSuccess;
-  // auxiliary stream: rhat transposed for the gains (estimated spectrum) or the gain pass
-  // (caller spectrum), overlapping the passes on the caller's stream
-  e = cudaEventRecord(p->ev_fork, s);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(p->aux, p->ev_fork, 0);
-  GainParams gp;
-  memset(&gp, 0, sizeof(gp));
-  gp.ny = p->ny; gp.L = p->L; gp.n_obs = p->n_obs; gp.n_un = p->n_un;
-  gp.spec = spectrum;
-  gp.rhat = rhat;
-  gp.goo = reinterpret_cast<float*>(ws + p->off_goo);
-  gp.gjo = reinterpret_cast<float2*>(ws + p->off_gjo);
-  gp.scale = (float)(1.0 / ((double)p->ny * (double)p->nx));
-  gp.status = p->d_status;
-  double* rhat_t = reinterpret_cast<double*>(ws + p->off_rhat_t);
-  if (spectrum && drawn) {   // the drawn perturbations scale by sqrt(rhat) in the column layout
-    prof_begin(p, kPassRhatT, p->aux);
-    if (e == cudaSuccess) e = launch_rhat_transpose(rhat, rhat_t, p->n_obs, p->ny, p->L, p->aux);
-    prof_end(p, kPassRhatT, p->aux);
-  }
-  const bool fused = !spectrum && p->use_fused();
-  float* amp_t = reinterpret_cast<float*>(ws + p->off_amp);
-  if (!spectrum) {
-    // the fused pass draws perturbations with the FP32 amplitudes sqrt(ny nx rhat) of the same pass
-    prof_begin(p, kPassRhatT, p->aux);
-    if (e == cudaSuccess)
-      e = launch_rhat_transpose(rhat, rhat_t, p->n_obs, p->ny, p->L, p->aux, (fused && drawn) ? amp_t : nullptr,
-                                (float)std::sqrt((double)p->ny * (double)p->nx));
-    prof_end(p, kPassRhatT, p->aux);
-  } else {
-    prof_begin(p, kPassGain, p->aux);
-    if (e == cudaSuccess) e = launch_gain(gp, p->aux);
-    prof_end(p, kPassGain, p->aux);
-  }
-  if (e == cudaSuccess) e = cudaEventRecord(p->ev_join, p->aux);
-  if (fused) {
-    // anomaly rows now; the columns after the innovation rows
-    if (e == cudaSuccess) e = run_anomaly_rows(p, ensemble, ws, s);
-  } else if (!spectrum && p->coupled) {
-    // tables of the column statistics, then the coupled gains (FP64 bracket inverse per wavenumber)
-    if (e == cudaSuccess) e = run_statistics(p, ensemble, ws, s, nullptr);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
-    CoupledGainParams cg;
-    memset(&cg, 0, sizeof(cg));
-    cg.ny = p->ny; cg.L = p->L; cg.n_obs = p->n_obs; cg.n_un = p->n_un; cg.n_pair = p->n_pair;
-    cg.chat_t = reinterpret_cast<const float*>(ws + p->off_chat);
-    cg.rhat_t = rhat_t;
-    cg.gall = gp.gjo;
-    cg.inv_G = (float)(1.0 / ((double)p->ny * (double)p->nx));
-    cg.status = p->d_status;
-    prof_begin(p, kPassGain, s);
-    if (e == cudaSuccess) e = launch_coupled_gain(cg, s);
-    prof_end(p, kPassGain, s);
-  } else if (!spectrum) {
-    // anomaly rows need no rhat; the statistics pass (which forms the gains) waits for it
-    if (e == cudaSuccess) e = run_statistics(p, ensemble, ws, s, rhat_t, p->ev_join);
-  } else {
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
-  }
-  RowFwdParams rp;
-  memset(&rp, 0, sizeof(rp));
-  rp.ny = p->ny; rp.nx = p->nx; rp.L = p->L; rp.M = p->M; rp.N = p->N;
-  rp.n_obs = p->n_obs; rp.mode = drawn ? kInnovationDrawn : kInnovation; rp.storage = p->storage;
-  for (int i = 0; i < p->n_obs; ++i) rp.obs[i] = p->obs[i];
-  rp.ens = ensemble; rp.data = data; rp.pert = perturbations;
-  rp.out = reinterpret_cast<float2*>(ws + p->off_W);
-  rp.vsel = p->sched[kPassRowInnov];
-  rp.twL = p->twL(rp.vsel & 1); rp.twX = p->twX(); rp.status = p->d_status;
-  prof_begin(p, kPassRowInnov, s);
-  if (e == cudaSuccess) e = launch_row_fwd(rp, p->N * p->n_obs, s);
-  prof_end(p, kPassRowInnov, s);
-  ColUpdParams up;
-  memset(&up, 0, sizeof(up));
-  up.ny = p->ny; up.L = p->L; up.M = p->M; up.N = p->N; up.n_obs = p->n_obs; up.n_un = p->n_un;
-  for (int j = 0; j < p->M; ++j) {
-    up.obs_of_block[j] = p->obs_of_block[j];
-    up.un_of_block[j] = p->un_of_block[j];
-  }
-  up.W = rp.out; up.goo = gp.goo; up.gjo = gp.gjo;
-  up.coupled = p->coupled ? 1 : 0;
-  up.gall = gp.gjo;
-  up.drawn = drawn ? 1 : 0;
-  up.seed = seed;
-  up.rhat_t = rhat_t;
-  up.sqrt_G = (float)std::sqrt((double)p->ny * (double)p->nx);
-  up.S = reinterpret_cast<float2*>(ws + p->off_A);
-  up.vsel = p->sched[kPassUpdate];
-  up.twY = p->twY(up.vsel); up.status = p->d_status;
-  if (fused) {
-    ColFusedParams f = fused_params(p, ws);
-    f.W = rp.out;
-    f.rhat_t = rhat_t;
-    f.drawn = drawn ? 1 : 0;
-    f.seed = seed;
-    f.amp_t = amp_t;
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
+  if (split & kSplitCols) {   // the columns read rhat or the caller's spectrum as they are
+    e = run_rows(p, q, !spectrum, innovations, split, ws, s);
+    q.spec = spectrum;
+    q.drawn = drawn ? 1 : 0;
+    q.seed = seed;
     prof_begin(p, kPassFused, s);
-    if (e == cudaSuccess) e = launch_col_fused(f, s);
+    if (e == cudaSuccess) e = launch_col_split(q, s);
     prof_end(p, kPassFused, s);
   } else {
-    prof_begin(p, kPassUpdate, s);
-    if (e == cudaSuccess) e = launch_col_update(up, s);
-    prof_end(p, kPassUpdate, s);
+    e = run_columns(p, q, spectrum, drawn, seed, split, ws, s);
   }
-  RowInvParams ip;
-  memset(&ip, 0, sizeof(ip));
-  ip.ny = p->ny; ip.nx = p->nx; ip.L = p->L; ip.M = p->M; ip.N = p->N; ip.storage = p->storage;
-  ip.vsel = p->sched[kPassRowInv];
-  ip.ens = ensemble; ip.twL = p->twL(ip.vsel & 1); ip.twX = p->twX(); ip.status = p->d_status;
-  ip.R = row_inv_rows(p->L, ip.vsel, p->ny, p->nx, p->storage == FFTENKF_BF16 ? 2 : 4);
-  // columns per tensor copy: the largest divisor of L that is at most 256
-  ip.box_cols = p->L < 256 ? p->L : 256;
-  while (p->L % ip.box_cols) --ip.box_cols;
-  if (p->tm_S != up.S || p->tm_R != ip.R) {   // re-encoded when the workspace or the item rows change
-    p->tm_ok = encode_increment_map(&p->tm, up.S, p->M * p->N, p->ny, p->L, ip.R, ip.box_cols);
-    p->tm_S = up.S;
-    p->tm_R = ip.R;
+  if (e == cudaSuccess && (split & kSplitInv)) {
+    prof_begin(p, kPassRowInv, s);
+    e = launch_row_inv_split(q, s);
+    prof_end(p, kPassRowInv, s);
+  } else if (e == cudaSuccess) {
+    RowInvParams ip;
+    memset(&ip, 0, sizeof(ip));
+    ip.ny = p->ny; ip.nx = p->nx; ip.L = p->L; ip.M = p->M; ip.N = p->N; ip.storage = p->storage;
+    ip.vsel = p->sched[kPassRowInv];
+    ip.ens = ensemble; ip.twL = p->twL(ip.vsel & 1); ip.twX = p->twX(); ip.status = p->d_status;
+    ip.R = row_inv_rows(p->L, ip.vsel, p->ny, p->nx, p->storage == FFTENKF_BF16 ? 2 : 4);
+    // columns per tensor copy: the largest divisor of L that is at most 256
+    ip.box_cols = p->L < 256 ? p->L : 256;
+    while (p->L % ip.box_cols) --ip.box_cols;
+    if (p->tm_S != q.one.A || p->tm_R != ip.R) {   // re-encoded when the workspace or the item rows change
+      p->tm_ok = encode_increment_map(&p->tm, q.one.A, p->M * p->N, p->ny, p->L, ip.R, ip.box_cols);
+      p->tm_S = q.one.A;
+      p->tm_R = ip.R;
+    }
+    if (!p->tm_ok) return fail(FFTENKF_ECUDA, "analyze: tensor map of the increment spectra refused");
+    ip.tm_in = p->tm;
+    prof_begin(p, kPassRowInv, s);
+    e = launch_row_inv(ip, p->M * p->N, s);
+    prof_end(p, kPassRowInv, s);
   }
-  if (!p->tm_ok && e == cudaSuccess) return fail(FFTENKF_ECUDA, "analyze: tensor map of the increment spectra refused");
-  ip.tm_in = p->tm;
-  prof_begin(p, kPassRowInv, s);
-  if (e == cudaSuccess) e = launch_row_inv(ip, p->M * p->N, s);
-  prof_end(p, kPassRowInv, s);
   if (e != cudaSuccess) return cuda_fail(e, "analyze");
   return FFTENKF_OK;
 }

@@ -192,6 +192,61 @@ cudaError_t launch_col_fused(const ColFusedParams& p, cudaStream_t s);
 // whether the fused column pass covers (ny, n_obs, blocks) with schedule sel
 bool col_fused_supported(int ny, int n_obs, int M, int sel);
 
+// The split passes (k_split.cuh): one analysis, or the analyses of one shape of a batch.
+struct SplitItem {
+  int N;
+  float inv_sqrt_N;       // 1 / sqrt(N)
+  float scale;            // 1 / ((N-1) ny nx)
+  void* ens;              // [M][N][ny][nx] storage dtype, updated in place
+  const float* data;      // [n_obs][ny][nx]
+  const void* pert;       // [N][n_obs][ny][nx] storage dtype
+  const double* rhat;     // [n_obs][ny][nx/2+1]
+  float2* A;              // anomaly row spectra, field j*N+k, then the increments
+  float2* W;              // innovation row spectra, field k*n_obs+i
+};
+struct SplitParams {
+  int ny, nx, L, M, n_obs, n_un, storage;
+  int obs[kMaxObs];
+  int role_block[kMaxBlocks];   // block of role r (r < n_obs: the observed ones)
+  SplitItem one;          // the item of an unbatched launch
+  const SplitItem* table; // batched: items, and the (item, unit) of every CTA
+  const uint2* units;
+  int n_units;
+  int anomalies;          // forward rows: the anomalies are transformed
+  int innovations;        // forward rows: 0, kInnovation or kInnovationDrawn
+  const float2 *twL, *twX, *twY;   // tables of split_row_V(L), plan_V(ny, split_col_sel)
+  int R;                  // rows per tile (set by split_row_shape)
+  int groups;             // thread groups of the column pass (set by split_col_shape)
+  int acc_bytes;          // shared memory of its sums
+  float* chat;            // columns: covariance tables wanted instead of the update, in the col_stats layout
+  const double* spec;     // columns: caller's spectrum tables in place of the sums
+  float inv_G;            // 1 / (ny nx)
+  int drawn;              // columns: perturbations drawn here under `seed`
+  unsigned long long seed;
+  float sqrt_G;
+  int* status;
+};
+// values per thread of the split passes' line plans: narrow lines have more threads
+__host__ __device__ constexpr int split_row_V(int L) {
+  return L % 3 == 0 ? (L >= 192 ? 24 : (L >= 12 ? 12 : L)) : (L >= 128 ? 16 : (L >= 8 ? 8 : L));
+}
+// line plan (plan_V selector) of the split columns: wide lines without cross sums, whose threads keep the
+// sums in registers; narrow ones for short lines and with cross sums
+__host__ __device__ constexpr int split_col_sel(int ny, bool cross) {
+  return (cross || (ny % 3 == 0 ? ny < 192 : (ny < 128 || ny == 512))) ? 1 : 0;
+}
+bool split_rows_supported(int L);
+bool split_cols_supported(int ny, int n_obs, int M);
+int split_row_tile(int L);                                    // rows per tile
+int split_col_groups(int ny, int n_obs, int M, int N);        // thread groups of one column's CTA
+cudaError_t launch_row_split(SplitParams p, cudaStream_t s);
+cudaError_t launch_col_split(SplitParams p, cudaStream_t s);
+cudaError_t launch_row_inv_split(SplitParams p, cudaStream_t s);
+
+// column groups that the fused pass keeps on the GPU at once
+int col_fused_groups(int ny, int sel);
+int sm_count();
+
 struct GainParams {
   int ny, L, n_obs, n_un;
   const float* chat_t;    // stats kernel output (transposed, float), or null

@@ -7,7 +7,7 @@
 // fully coalesced warp accesses, and a forward transform's output can feed an
 // inverse transform without any exchange.  Between radix stages the values go
 // through a padded shared-memory line buffer (Stockham self-sorting order), so
-// no bit reversal is needed.  Radices are 16, 8, 4, 2 and 3; the plan is fixed
+// no bit reversal is needed.  Radices are 24, 16, 12, 8, 6, 4, 3 and 2; the plan is fixed
 // at compile time from (N, V).
 #pragma once
 #include <cuda_runtime.h>
@@ -33,8 +33,16 @@ __device__ __forceinline__ float2 rot90(float2 a) {
 }
 
 // ------------------------------------------------------------------ plan
+// Radix of the next stage of a line with `rem` left, V values per thread.  3 * 2^a lines take the factor
+// 3 together with a power of two (radices 6, 12 and 24), so that it costs no exchange of its own: 24
+// first, where it leaves stages of 8 and at most one of 4, otherwise last as 6 (384 = 8 8 6; V = 12:
+// 12 first or 6 last, as the power of two is even or odd).
 __host__ __device__ constexpr int pick_radix(int rem, int V) {
-  return (rem % 16 == 0 && V % 16 == 0) ? 16
+  return (V == 24 && (rem == 24 || rem == 96 || rem == 192 || rem == 768 || rem == 1536)) ? 24
+       : (V == 24 && rem == 6)          ? 6
+       : (V == 12 && (rem == 12 || rem == 48 || rem == 192 || rem == 768 || rem == 3072)) ? 12
+       : (V == 12 && rem == 6)          ? 6
+       : (rem % 16 == 0 && V % 16 == 0) ? 16
        : (rem % 8 == 0 && V % 8 == 0)   ? 8
        : (rem % 4 == 0 && V % 4 == 0)   ? 4
        : (rem % 2 == 0 && V % 2 == 0)   ? 2
@@ -186,15 +194,40 @@ template <bool INV> struct Dft<16, INV> {
   }
 };
 
+// 3 P-point DFT (P = 2, 4, 8) from P-point and 3-point ones without twiddles between them (Good's prime
+// factor map): input 3 n1 + P n2, output K1 k1 + K2 k2 (mod 3 P), K1 = 1 mod P and 0 mod 3, K2 the reverse
+template <int P, bool INV> struct DftPrime3 {
+  static __device__ __forceinline__ void run(float2* a) {
+    constexpr int K1 = (P == 2) ? 3 : 9, K2 = (P == 8) ? 16 : 4;
+    float2 y[3][P];
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < P; ++n1) y[n2][n1] = a[(3 * n1 + P * n2) % (3 * P)];
+      Dft<P, INV>::run(y[n2]);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < P; ++k1) {
+      float2 t[3] = {y[0][k1], y[1][k1], y[2][k1]};
+      Dft<3, INV>::run(t);
+#pragma unroll
+      for (int k2 = 0; k2 < 3; ++k2) a[(K1 * k1 + K2 * k2) % (3 * P)] = t[k2];
+    }
+  }
+};
+template <bool INV> struct Dft<6, INV> : DftPrime3<2, INV> {};
+template <bool INV> struct Dft<12, INV> : DftPrime3<4, INV> {};
+template <bool INV> struct Dft<24, INV> : DftPrime3<8, INV> {};
+
 // Twiddle tables.  Butterfly j of a stage with NS > 1 multiplies its input r by w^r,
 // w = W_N^((j mod NS) N/(NS R)).  The table stores only the powers w^p for p in
-// {1, 2, 4, 8} below R (w and w^2 for radix 3), as rows of NS entries (the threads of a
+// {1, 2, 4, 8, 16} below R (w and w^2 for radix 3), as rows of NS entries (the threads of a
 // warp, consecutive j, read consecutive entries); the butterfly forms the other powers
 // by at most three complex products (w^3 = w^2 w, w^5 = w^4 w, ..., w^15 = w^8 w^7).
 // A 4096-point plan then needs 1088 entries (8.5 KB) instead of 4080, which stay in L1
 // when a pass gives most of the SM's on-chip memory to shared memory.  Stages are
 // concatenated in order; twiddle_offset(N, V, s) is where stage s starts.
-__host__ __device__ constexpr int tw_npow(int R) { return R == 16 ? 4 : R == 8 ? 3 : R == 4 ? 2 : R == 3 ? 2 : 1; }
+__host__ __device__ constexpr int tw_npow(int R) { return R > 16 ? 5 : R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : 1; }
 __host__ __device__ constexpr int tw_pow(int q) { return 1 << q; }   // the q-th stored power
 __host__ __device__ constexpr int stage_ns(int N, int V, int s) {
   int ns = 1;
@@ -231,7 +264,7 @@ __device__ __forceinline__ void twiddle_powers(float2 (&w)[R], const float2* __r
 #pragma unroll
   for (int r = 3; r < R; ++r) {
     if ((r & (r - 1)) == 0) continue;          // stored
-    const int hi = r >= 8 ? 8 : (r >= 4 ? 4 : 2);   // largest stored power below r
+    const int hi = r >= 16 ? 16 : (r >= 8 ? 8 : (r >= 4 ? 4 : 2));   // largest stored power below r
     w[r] = cmul(w[hi], w[r - hi]);
   }
 }
@@ -250,11 +283,12 @@ __device__ __forceinline__ void line_sync(int bid) {
     asm volatile("bar.sync %0, %1;" ::"r"(bid), "n"(T) : "memory");
   }
 }
-// barrier id of line group g for line_sync: 1 + g when lines of T threads own whole warps
-// (at most 8 lines per CTA of up to 512 threads), else 0 (the CTA barrier)
+// barrier id of line group g for line_sync: the line's own warp when a line is at most one warp
+// (T divides 32, so no line straddles two warps), 1 + g when lines of T threads own several whole
+// warps (at most 8 lines per CTA of up to 512 threads), else 0 (the CTA barrier)
 template <int T>
 __device__ __forceinline__ int line_bar(int g) {
-  return (T % 32 == 0 && T >= 64) ? 1 + g : 0;
+  return (32 % T == 0) ? -1 : (T % 32 == 0) ? 1 + g : 0;
 }
 
 // ------------------------------------------------------------------ stages

@@ -105,6 +105,8 @@ bool col_fused_supported(int ny, int n_obs, int M, int sel) {
   return (nf + 4) * s.V <= s.cols_per_thread;     // + the member's spectra (two complex halves)
 }
 
+int col_fused_groups(int ny, int sel) { return sm_count() * col_fused_launch(ny, sel).lpc; }
+
 cudaError_t launch_col_fused(const ColFusedParams& p, cudaStream_t s) {
   if (!col_fused_supported(p.ny, p.n_obs, p.M, p.vsel)) return cudaErrorNotSupported;
   return p.n_obs == 1 ? col_fused_nobs1(p, s) : col_fused_nobs2(p, s);

@@ -1,0 +1,6 @@
+// Split column pass, instantiated for up to 4 observed block(s).
+#include "k_split.cuh"
+
+namespace fftenkf {
+cudaError_t col_split_4(const SplitParams& p, int units, cudaStream_t s) { return col_split_dispatch<4, false>(p, units, s); }
+}  // namespace fftenkf

@@ -1,0 +1,42 @@
+// Kernel launches of the analysis passes: shape look-ups made once per (device, kernel, shape), and
+// launches that may overlap the tail of the kernel before them (programmatic dependent launch).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace fftenkf {
+
+// Resident CTAs per SM of `kern` with `threads` and `smem` bytes of dynamic shared memory, after
+// allowing it that much.  The attribute call and the occupancy query cost several microseconds of host
+// time, more than a launch, so the answers are kept, one entry per (device, kernel, threads, smem)
+// that was ever launched.
+cudaError_t kernel_shape(const void* kern, int threads, size_t smem, int* per_sm);
+
+// In a kernel launched with launch_overlapped: returns once every earlier kernel of the stream has
+// finished and its writes are visible; nothing of an earlier kernel is read or overwritten before it.
+// Data of earlier kernels is read by plain loads: the compiler may move __ldg and loads through const
+// __restrict__ pointers, which it takes for loads of constants, ahead of this wait.
+// It then lets the next kernel of the stream be brought onto SMs that have room, where it waits here.
+__device__ __forceinline__ void stream_order_wait() {
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch with the stream's order kept by stream_order_wait() at the kernel's start: the launch latency
+// of a kernel overlaps the one before it (2-3 us between dependent kernels otherwise).
+template <typename P>
+inline cudaError_t launch_overlapped(void (*kern)(const P), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                     const P& p) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+}  // namespace fftenkf

@@ -297,7 +297,8 @@ struct MlpBins {
   const uint32_t* seg_off;   // [nseg + 1] segment offsets into order (each within one bin)
   const uint32_t* bin_seg;   // [129] first segment of every bin
   const float* centre_log;   // [128]
-  unsigned* cmax_bits;       // [max_batch] scratch
+  float* cmax;               // [max_batch][chunks] scratch
+  int chunks;
   float* part;               // [max_batch][nseg] scratch
 };
 

@@ -11,10 +11,11 @@ namespace fftenkf {
 void set_last_error(const std::string& msg);
 int mlp_param_count();
 int mlp_seg_len();
+int mlp_chunks(int K1);
 cudaError_t launch_mlp_bin(const double* chat, const MlpBins& t, int B, float* feat, float* mean, cudaStream_t s);
-cudaError_t launch_mlp_finish(const float* out, const float* mean, float* out_log, int* flag, const double* chat_in,
-                              double* chat_out, int K1, int ny, int L, float w, cudaStream_t s);
-cudaError_t launch_mlp_forward(const float* params, const float* X, int B, float* out, float* acts, cudaStream_t s);
+cudaError_t launch_mlp_denoise(const double* chat_in, const MlpBins& t, const float* params, float* out_log, int* flag,
+                               double* chat_out, int ny, int L, float w, cudaStream_t s);
+cudaError_t launch_mlp_forward(const float* params, const float* X, int B, float* out, cudaStream_t s);
 cudaError_t launch_mlp_gradient(const float* params, const float* X, const float* target, int B, float* grads,
                                 float* loss, cudaStream_t s);
 cudaError_t launch_mlp_adam(float* params, float* m, float* v, const float* g, int step, float lr, cudaStream_t s);
@@ -42,12 +43,12 @@ struct fftenkf_denoiser_s {
   uint32_t* d_seg = nullptr;     // segment offsets [nseg + 1] | first segment of every bin [129]
   int nseg = 0;
   float* d_centre_log = nullptr;
-  float* d_scratch = nullptr;   // features 256 | mean 1 | out 128 | out_log 128
-  unsigned* d_cmax = nullptr;   // [kMaxBatch]
+  float* d_scratch = nullptr;   // out_log [128]
+  float* d_cmax = nullptr;      // [kMaxBatch][chunks]
   float* d_part = nullptr;      // [kMaxBatch][nseg]
   int* d_flag = nullptr;
   MlpBins bins() const {
-    return MlpBins{K1, nseg, kMaxBatch, d_order, d_start, d_seg, d_seg + nseg + 1, d_centre_log, d_cmax, d_part};
+    return MlpBins{K1, nseg, kMaxBatch, d_order, d_start, d_seg, d_seg + nseg + 1, d_centre_log, d_cmax, mlp_chunks(K1), d_part};
   }
 };
 
@@ -102,11 +103,11 @@ extern "C" fftenkf_status fftenkf_denoiser_create(fftenkf_denoiser* out, int ny,
   if (e == cudaSuccess) e = cudaMemcpy(d->d_start, start.data(), (kNB + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&d->d_seg, seg.size() * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemcpy(d->d_seg, seg.data(), seg.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&d->d_cmax, kMaxBatch * sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMalloc(&d->d_cmax, (size_t)kMaxBatch * mlp_chunks(d->K1) * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&d->d_part, (size_t)kMaxBatch * std::max(d->nseg, 1) * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&d->d_centre_log, kNB * sizeof(float));
   if (e == cudaSuccess) e = cudaMemcpy(d->d_centre_log, cl.data(), kNB * sizeof(float), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&d->d_scratch, (256 + 4 + 2 * kNB) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&d->d_scratch, kNB * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&d->d_flag, sizeof(int));
   if (e != cudaSuccess) {
     fftenkf_denoiser_destroy(d);
@@ -142,7 +143,7 @@ extern "C" fftenkf_status fftenkf_mlp_forward(const float* params, const float* 
                                               void* stream) {
   set_last_error("");
   if (!params || !features || !out || batch <= 0) return mfail(FFTENKF_EINVAL, "bad arguments");
-  return mcuda(launch_mlp_forward(params, features, batch, out, nullptr, static_cast<cudaStream_t>(stream)),
+  return mcuda(launch_mlp_forward(params, features, batch, out, static_cast<cudaStream_t>(stream)),
                "mlp_forward");
 }
 
@@ -171,14 +172,7 @@ extern "C" fftenkf_status fftenkf_denoise_spectrum(fftenkf_denoiser d, const flo
     if (used_fallback) *used_fallback = 1;
     return mcuda(e, "denoise_spectrum");
   }
-  float* feat = d->d_scratch;
-  float* mean = feat + 256;
-  float* out = mean + 4;
-  float* out_log = out + kNB;
-  cudaError_t e = launch_mlp_bin(chat_in, d->bins(), 1, feat, mean, s);
-  if (e == cudaSuccess) e = launch_mlp_forward(params, feat, 1, out, nullptr, s);
-  if (e == cudaSuccess)
-    e = launch_mlp_finish(out, mean, out_log, d->d_flag, chat_in, chat_out, d->K1, d->ny, d->L, d->w, s);
+  cudaError_t e = launch_mlp_denoise(chat_in, d->bins(), params, d->d_scratch, d->d_flag, chat_out, d->ny, d->L, d->w, s);
   if (e != cudaSuccess) return mcuda(e, "denoise_spectrum");
   if (used_fallback) {
     e = cudaMemcpyAsync(used_fallback, d->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s);

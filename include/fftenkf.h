@@ -230,14 +230,13 @@ fftenkf_status fftenkf_set_coupled(fftenkf_plan plan, int coupled);
 /* ---------------------------------------------------------------- batched
  * Many independent analyses of uneven sizes (the block-state method with one
  * fully observed block each, H = I, eq. spectral-enkf), replayed as one CUDA
- * graph (captured on the first call, after every autotune, and when the
- * pointers of an analysis of at least 512 x 256 points change).  Analyses of at
- * least 512 x 256 grid points run through the single-analysis passes (one plan
- * each, created with the batch), issued on eight graph branches, largest first,
- * each to the branch with the least work; every other analysis goes through
- * seven persistent launches, each over a work list mixing the units of all of
- * them, on a branch of its own.  dims[i].n_blocks must be 1; all analyses
- * share one storage type; ny and nx/2 in {2^a, 3*2^a} between 16 and 1024.
+ * graph (captured on the first call and after every autotune).  Analyses of one
+ * grid shape share their launches: forward rows, columns, inverse rows, each over
+ * the units of all of them; the shapes run on eight graph branches, largest first,
+ * each on the branch with the least work.  The kernels read the pointers of an
+ * analysis from a device table, so new pointers cost one table copy and no new
+ * capture.  dims[i].n_blocks must be 1; all analyses share one storage type; ny
+ * and nx/2 in {2^a, 3*2^a} between 16 and 1024.
  * The pointer arguments of fftenkf_analyze_batched are HOST arrays of `count`
  * DEVICE pointers with the single-analysis layouts (ensemble [N][ny][nx],
  * data [ny][nx] float, perturbations [N][ny][nx], rhat [ny][nx/2+1] double). */
@@ -248,13 +247,14 @@ fftenkf_status fftenkf_batch_workspace_size(fftenkf_batch batch, size_t* bytes);
 fftenkf_status fftenkf_analyze_batched(fftenkf_batch batch, void* const* ensembles, const float* const* data,
                                        const void* const* perturbations, const double* const* rhat,
                                        void* workspace, void* stream);
-/* Autotuner: times every candidate CTA size (128, 256 threads) and line-FFT
- * schedule (0, 1) of every pass on zero-filled scratch inputs of the batch's
+/* Autotuner: times every candidate CTA size (128, 256 threads) of the forward
+ * rows, columns and inverse rows on zero-filled scratch inputs of the batch's
  * shapes (allocated for the call: one copy of every item's inputs) and keeps
  * the fastest; best_ms (may be NULL) receives the sum of the best pass times. */
 fftenkf_status fftenkf_batch_autotune(fftenkf_batch batch, void* workspace, void* stream, double* best_ms);
 /* Chosen CTA size and schedule of each batched pass (7 passes: mean, anomaly
- * rows, statistics, gain, innovation rows, update, inverse rows). */
+ * rows, statistics, gain, innovation rows, update, inverse rows; passes that share
+ * a launch report the same, and the schedule is always 0). */
 fftenkf_status fftenkf_batch_schedule(fftenkf_batch batch, int* cta_threads, int* sched, int n);
 fftenkf_status fftenkf_batch_last_device_status(fftenkf_batch batch, void* stream);
 

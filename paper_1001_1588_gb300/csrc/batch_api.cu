@@ -1,29 +1,29 @@
-// C ABI of the batched analyses: plan (work lists, workspace layout, twiddle
-// tables), autotuner (CTA size and line-FFT schedule per pass, chosen by
-// timing the candidates on scratch data of the batch's shapes), and the
+// C ABI of the batched analyses: plan (shape classes, item table, unit lists, workspace layout, twiddle
+// tables), autotuner (CTA sizes of the passes, timed on scratch data of the batch's shapes), and the
 // analysis itself, replayed as one CUDA graph.
 //
-// Analyses of at least kBigPoints grid points run through the single-analysis
-// passes (one plan each, whose pipelined row and column kernels move their
-// bytes at several times the rate of the persistent batched passes); they are
-// issued on kLanes streams that branch off the capture (largest first, each to
-// the lane with the least work so far), beside the seven persistent launches
-// that take every smaller analysis, so that the branches fill the GPU together.
+// Items of one grid shape form a class.  A class runs the split passes (k_split.cuh) with one launch per
+// pass over the units of its items: forward rows (anomalies and innovations), columns, inverse rows.  The
+// kernels take the pointers of an item from a device table, so that new pointers need a new table and no
+// new graph.  Classes are cut into chunks of at most kChunkBytes of their working set and issued on
+// kLanes graph branches, largest first, each to the branch with the least work.  (256 mixed analyses, 8 to
+// 1024 points a side, FP32: 12.32 -> 8.16 ms.  Before, the 103 analyses of at least 512 x 256 points ran on
+// plans of their own, whose kernels each filled a fraction of the SMs, and the others in seven persistent
+// launches whose units were serial over the members.)
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/fftenkf.h"
-#include "batch.cuh"
-#include "k_batch.cuh"
+#include "common.cuh"
 
 using namespace fftenkf;
 
 namespace fftenkf {
-int sm_count();
 void set_last_error(const std::string& msg);
 }  // namespace fftenkf
 
@@ -33,145 +33,137 @@ fftenkf_status bfail(fftenkf_status s, const std::string& m) {
   return s;
 }
 size_t rup(size_t x, size_t a) { return (x + a - 1) / a * a; }
-const int kCandBt[2] = {128, 256};
-#ifndef FFTENKF_BATCH_BIG_POINTS
-#define FFTENKF_BATCH_BIG_POINTS (512LL * 256)
-#endif
-#ifndef FFTENKF_BATCH_LANES
-#define FFTENKF_BATCH_LANES 8
-#endif
-constexpr long long kBigPoints = FFTENKF_BATCH_BIG_POINTS;   // grid points from which an analysis takes its own plan
-constexpr int kLanes = FFTENKF_BATCH_LANES;
+constexpr int kLanes = 8;
+constexpr size_t kChunkBytes = (size_t)1 << 40;
+constexpr int kBatchPasses = 7;   // reported passes: mean, anomaly rows, statistics, gain, innovation rows, update, inverse rows
+enum Stage { kRows, kCols, kInv, kStages };
+// the stage that a reported pass is part of
+Stage stage_of(int pass) { return (pass == 1 || pass == 4) ? kRows : (pass == 6) ? kInv : kCols; }
+const int kCandBt[2] = {256, 128};
+
+bool batch_line(int n) { return n >= 16 && n <= 1024 && line_supported(n) && row_line_supported(n); }
+
+struct Chunk {
+  int ny, nx, n_max;            // shape, largest member count
+  double cost;
+  int first[kStages], units[kStages];   // its units in the unit list of the batch
+};
 }  // namespace
 
 struct fftenkf_batch_s {
   int count = 0, storage = 0;
-  std::vector<BatchItem> items;              // host copy (pointers of the last bound call)
-  BatchItem* d_items = nullptr;
+  std::vector<fftenkf_dims> dims;
+  std::vector<SplitItem> items;        // host copy (pointers of the last bound call)
+  std::vector<size_t> off_A, off_W;    // workspace regions
+  std::vector<Chunk> chunks;           // largest first
+  SplitItem* d_items = nullptr;
+  uint2* d_units = nullptr;
   float2* d_tw = nullptr;
+  std::map<std::pair<int, int>, size_t> off_tw;   // (line length, V) -> stage twiddles
+  std::map<int, size_t> off_x;                    // nx -> real-FFT twiddles
   int* d_status = nullptr;
   size_t ws_bytes = 0;
   void* own_ws = nullptr;
-  std::vector<size_t> off_mean, off_A, off_W, off_chat, off_gain;
-  // per-pass launch configuration
-  int bt[kBPassCount], vsel[kBPassCount];
-  BatchUnit* d_units[kBPassCount] = {};
-  int n_units[kBPassCount] = {};
-  size_t smem[kBPassCount] = {};
-  int grid[kBPassCount] = {};
-  // analyses on their own plans (null: in the batched passes), their workspace regions
-  std::vector<fftenkf_plan> sub;
-  std::vector<size_t> off_sub;
+  int bt[kStages] = {256, 256, 256};
   cudaStream_t lane[kLanes] = {};
   cudaEvent_t ev_fork = nullptr, ev_lane[kLanes] = {};
-  // graph of the launches
   cudaStream_t cap = nullptr;
   cudaGraphExec_t exec = nullptr;
   char* bound_ws = nullptr;
   bool items_dirty = true;
-  bool sub_dirty = true;   // pointers of a planned analysis changed: capture again
 };
 
-// work list and launch shape of pass `pass` for CTA size bt and schedule vsel
-static fftenkf_status build_pass(fftenkf_batch b, int pass, int bt, int vsel) {
-  struct U {
-    double cost;
-    BatchUnit u;
+static SplitParams chunk_params(fftenkf_batch b, const Chunk& c) {
+  SplitParams q;
+  memset(&q, 0, sizeof(q));
+  q.ny = c.ny; q.nx = c.nx; q.L = c.nx / 2; q.M = 1; q.n_obs = 1; q.storage = b->storage;
+  q.table = b->d_items;
+  q.anomalies = 1;
+  q.innovations = kInnovation;
+  q.twL = b->d_tw + b->off_tw[{q.L, split_row_V(q.L)}];
+  q.twX = b->d_tw + b->off_x[c.nx];
+  q.twY = b->d_tw + b->off_tw[{c.ny, plan_V(c.ny, split_col_sel(c.ny, false))}];
+  q.inv_G = (float)(1.0 / ((double)c.ny * (double)c.nx));
+  q.status = b->d_status;
+  return q;
+}
+
+static cudaError_t run_stage(fftenkf_batch b, const Chunk& c, int stage, cudaStream_t s) {
+  SplitParams q = chunk_params(b, c);
+  q.units = b->d_units + c.first[stage];
+  q.n_units = c.units[stage];
+  q.threads = b->bt[stage];
+  if (stage == kRows) return launch_row_split(q, s);
+  if (stage == kInv) return launch_row_inv_split(q, s);
+  q.groups = split_col_groups(c.ny, 1, 1, c.n_max, q.threads);
+  return launch_col_split(q, s);
+}
+
+// The whole batch on stream s: the chunks on the lanes, forked from s and joined back.
+static fftenkf_status run_all(fftenkf_batch b, cudaStream_t s) {
+  const int lanes = std::min((int)b->chunks.size(), kLanes);
+  cudaError_t e = cudaEventRecord(b->ev_fork, s);
+  double load[kLanes] = {};
+  for (int l = 0; l < lanes && e == cudaSuccess; ++l) e = cudaStreamWaitEvent(b->lane[l], b->ev_fork, 0);
+  for (const Chunk& c : b->chunks) {
+    int l = 0;
+    for (int q = 1; q < lanes; ++q)
+      if (load[q] < load[l]) l = q;
+    load[l] += c.cost;
+    for (int stage = 0; stage < kStages && e == cudaSuccess; ++stage) e = run_stage(b, c, stage, b->lane[l]);
+  }
+  for (int l = 0; l < lanes && e == cudaSuccess; ++l) {
+    e = cudaEventRecord(b->ev_lane[l], b->lane[l]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b->ev_lane[l], 0);
+  }
+  return e == cudaSuccess ? FFTENKF_OK : bfail(FFTENKF_ECUDA, std::string("batched passes: ") + cudaGetErrorString(e));
+}
+
+// Classes, chunks, unit lists (uploaded) and the workspace layout.
+static cudaError_t build_units(fftenkf_batch b) {
+  std::map<std::pair<int, int>, std::vector<int>> classes;
+  for (int i = 0; i < b->count; ++i) classes[{b->dims[i].ny, b->dims[i].nx}].push_back(i);
+  std::vector<uint2> units;
+  auto add_chunk = [&](int ny, int nx, const std::vector<int>& ids) {
+    Chunk c{};
+    c.ny = ny;
+    c.nx = nx;
+    const unsigned tiles = (unsigned)(ny / split_row_tile(nx / 2));
+    for (int i : ids) {
+      c.n_max = std::max(c.n_max, b->dims[i].n_members);
+      c.cost += (double)b->dims[i].n_members * ny * nx;
+    }
+    for (int stage = 0; stage < kStages; ++stage) {
+      c.first[stage] = (int)units.size();
+      for (int i : ids) {
+        const unsigned N = (unsigned)b->dims[i].n_members;
+        const unsigned n = stage == kRows ? 2 * N * tiles : stage == kInv ? N * tiles : (unsigned)(nx / 2 + 1);
+        for (unsigned u = 0; u < n; ++u) units.push_back(make_uint2((unsigned)i, u));
+      }
+      c.units[stage] = (int)units.size() - c.first[stage];
+    }
+    b->chunks.push_back(c);
   };
-  std::vector<U> list;
-  size_t smem = 0;
-  for (int i = 0; i < b->count; ++i) {
-    if (b->sub[i]) continue;   // on its own plan
-    const BatchItem& it = b->items[i];
-    const int n = batch_units(pass, it, bt, vsel);
-    const double c = batch_unit_cost(pass, it, bt, vsel);
-    for (int u = 0; u < n; ++u) list.push_back({c, {i, u}});
-    smem = std::max(smem, batch_smem(pass, it, bt, vsel));
-  }
-  if (smem > 200 * 1024) return bfail(FFTENKF_EUNSUPPORTED, "batched unit exceeds shared memory");
-  std::stable_sort(list.begin(), list.end(), [](const U& a, const U& c) { return a.cost > c.cost; });
-  std::vector<BatchUnit> units(list.size());
-  for (size_t i = 0; i < list.size(); ++i) units[i] = list[i].u;
-  if (b->d_units[pass]) cudaFree(b->d_units[pass]);
-  b->d_units[pass] = nullptr;
-  if (!units.empty()) {
-    if (cudaMalloc(&b->d_units[pass], units.size() * sizeof(BatchUnit)) != cudaSuccess)
-      return bfail(FFTENKF_ENOMEM, "work list allocation failed");
-    cudaMemcpy(b->d_units[pass], units.data(), units.size() * sizeof(BatchUnit), cudaMemcpyHostToDevice);
-  }
-  b->n_units[pass] = (int)units.size();
-  b->bt[pass] = (pass == kBGain) ? 256 : bt;
-  b->vsel[pass] = vsel;
-  b->smem[pass] = smem;
-  // persistent grid: as many CTAs as fit on the GPU at this shared memory size
-  const int by_smem = smem ? (int)((220 * 1024) / (smem + 1024)) : 16;
-  int per_sm = std::max(1, std::min(by_smem, 2048 / b->bt[pass]));
-  b->grid[pass] = std::max(1, std::min((int)units.size(), sm_count() * per_sm));
-  if (b->exec) {
-    cudaGraphExecDestroy(b->exec);
-    b->exec = nullptr;
-  }
-  return FFTENKF_OK;
-}
-
-static BatchParams pass_params(fftenkf_batch b, int pass) {
-  BatchParams p;
-  p.items = b->d_items;
-  p.units = b->d_units[pass];
-  p.n_units = b->n_units[pass];
-  p.storage = b->storage;
-  p.mode = (pass == kBRowInnov) ? kInnovation : kAnomaly;
-  p.vsel = b->vsel[pass];
-  p.status = b->d_status;
-  return p;
-}
-
-static cudaError_t run_passes(fftenkf_batch b, cudaStream_t s) {
-  for (int pass = 0; pass < kBPassCount; ++pass) {
-    if (b->n_units[pass] == 0) continue;   // every analysis on its own plan
-    cudaError_t e = launch_batch_pass(pass, pass_params(b, pass), b->bt[pass], b->smem[pass], b->grid[pass], s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-// The whole batch on stream s: the planned analyses on the lanes (forked from s and joined
-// back), the persistent passes of the others on s.
-static fftenkf_status run_all(fftenkf_batch b, void* const* ens, const float* const* data, const void* const* pert,
-                              const double* const* rhat, char* ws, cudaStream_t s) {
-  bool any = false;
-  for (int i = 0; i < b->count; ++i) any |= b->sub[i] != nullptr;
-  cudaError_t e = cudaSuccess;
-  if (any) {
-    e = cudaEventRecord(b->ev_fork, s);
-    for (int l = 0; l < kLanes && e == cudaSuccess; ++l) e = cudaStreamWaitEvent(b->lane[l], b->ev_fork, 0);
-    if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("fork: ") + cudaGetErrorString(e));
-    std::vector<int> order;
-    for (int i = 0; i < b->count; ++i)
-      if (b->sub[i]) order.push_back(i);
-    auto cost = [&](int i) { return (double)b->items[i].N * b->items[i].ny * b->items[i].nx; };
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
-    double load[kLanes] = {};
-    for (int i : order) {
-      int l = 0;
-      for (int q = 1; q < kLanes; ++q)
-        if (load[q] < load[l]) l = q;
-      load[l] += cost(i);
-      fftenkf_status st = fftenkf_analyze(b->sub[i], ens[i], data[i], pert[i], rhat[i], nullptr, ws + b->off_sub[i],
-                                          b->lane[l]);
-      if (st != FFTENKF_OK) return st;
+  for (auto& cl : classes) {
+    const int ny = cl.first.first, nx = cl.first.second;
+    std::vector<int> ids;
+    size_t bytes = 0;
+    for (int i : cl.second) {
+      const size_t w = (size_t)b->dims[i].n_members * ny * nx * 16;   // members, perturbations and both row spectra
+      if (!ids.empty() && bytes + w > kChunkBytes) {
+        add_chunk(ny, nx, ids);
+        ids.clear();
+        bytes = 0;
+      }
+      ids.push_back(i);
+      bytes += w;
     }
+    add_chunk(ny, nx, ids);
   }
-  e = run_passes(b, s);
-  if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("batched passes: ") + cudaGetErrorString(e));
-  if (any) {
-    for (int l = 0; l < kLanes && e == cudaSuccess; ++l) {
-      e = cudaEventRecord(b->ev_lane[l], b->lane[l]);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b->ev_lane[l], 0);
-    }
-    if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("join: ") + cudaGetErrorString(e));
-  }
-  return FFTENKF_OK;
+  std::stable_sort(b->chunks.begin(), b->chunks.end(), [](const Chunk& x, const Chunk& y) { return x.cost > y.cost; });
+  cudaError_t e = cudaMalloc(&b->d_units, units.size() * sizeof(uint2));
+  if (e == cudaSuccess) e = cudaMemcpy(b->d_units, units.data(), units.size() * sizeof(uint2), cudaMemcpyHostToDevice);
+  return e;
 }
 
 extern "C" fftenkf_status fftenkf_plan_batched(fftenkf_batch* out, int count, const fftenkf_dims* dims) {
@@ -185,110 +177,63 @@ extern "C" fftenkf_status fftenkf_plan_batched(fftenkf_batch* out, int count, co
     if (d.storage != storage) return bfail(FFTENKF_EINVAL, "all batched analyses share one storage type");
     if (d.storage != FFTENKF_F32 && d.storage != FFTENKF_BF16) return bfail(FFTENKF_EINVAL, "unknown storage");
     if (d.n_members < 2) return bfail(FFTENKF_EUNSUPPORTED, "need at least 2 members");
-    if (d.nx % 2 || !batch_line_supported(d.nx / 2) || !batch_line_supported(d.ny))
+    if (d.nx % 2 || !batch_line(d.nx / 2) || !batch_line(d.ny))
       return bfail(FFTENKF_EUNSUPPORTED, "batched sizes: ny and nx/2 in {2^a, 3*2^a} between 16 and 1024");
   }
   fftenkf_batch b = new fftenkf_batch_s();
   b->count = count;
   b->storage = storage;
+  b->dims.assign(dims, dims + count);
   b->items.resize(count);
-  // twiddle tables, one set per distinct line length
+  // twiddle tables, one per distinct line plan
   std::vector<float2> tw;
-  std::map<int, size_t> off_stage[2];
-  std::map<int, size_t> off_x;
-  auto stage_table = [&](int n, int sel) {
-    if (off_stage[sel].count(n)) return;
-    off_stage[sel][n] = tw.size();
-    const int V = plan_V(n, sel);
-    for (int i = 0; i < twiddle_count(n, V); ++i) {
-      const double ang = 2.0 * M_PI * (double)twiddle_exponent(n, V, i) / (double)n;
-      tw.push_back(make_float2((float)std::cos(ang), (float)-std::sin(ang)));
-    }
+  auto root = [&](long long e, long long n) {
+    const double ang = 2.0 * M_PI * (double)e / (double)n;
+    tw.push_back(make_float2((float)std::cos(ang), (float)-std::sin(ang)));
+  };
+  auto stage_table = [&](int n, int V) {
+    if (b->off_tw.count({n, V})) return;
+    b->off_tw[{n, V}] = tw.size();
+    for (int i = 0; i < twiddle_count(n, V); ++i) root(twiddle_exponent(n, V, i), n);
     if (tw.size() % 2) tw.push_back(make_float2(0.f, 0.f));
   };
+  size_t off = 0;
+  b->off_A.resize(count);
+  b->off_W.resize(count);
   for (int i = 0; i < count; ++i) {
-    const int L = dims[i].nx / 2, ny = dims[i].ny;
-    for (int sel = 0; sel < 2; ++sel) {
-      stage_table(L, sel);
-      stage_table(ny, sel);
-    }
-    if (!off_x.count(dims[i].nx)) {
-      off_x[dims[i].nx] = tw.size();
-      for (int k = 0; k <= L; ++k) {
-        const double ang = 2.0 * M_PI * (double)k / (double)dims[i].nx;
-        tw.push_back(make_float2((float)std::cos(ang), (float)-std::sin(ang)));
-      }
+    const int ny = dims[i].ny, nx = dims[i].nx, L = nx / 2, N = dims[i].n_members;
+    stage_table(L, split_row_V(L));
+    stage_table(ny, plan_V(ny, split_col_sel(ny, false)));
+    if (!b->off_x.count(nx)) {
+      b->off_x[nx] = tw.size();
+      for (int k = 0; k <= L; ++k) root(k, nx);
       if (tw.size() % 2) tw.push_back(make_float2(0.f, 0.f));
     }
+    SplitItem& it = b->items[i];
+    memset(&it, 0, sizeof(it));
+    it.N = N;
+    it.inv_sqrt_N = (float)(1.0 / std::sqrt((double)N));
+    it.scale = (float)(1.0 / ((double)(N - 1) * (double)ny * (double)nx));
+    const size_t lines = (size_t)N * L * ny * sizeof(float2);
+    b->off_A[i] = off; off = rup(off + lines, 256);
+    b->off_W[i] = off; off = rup(off + lines, 256);
   }
+  b->ws_bytes = off;
   cudaError_t e = cudaMalloc(&b->d_tw, tw.size() * sizeof(float2));
   if (e == cudaSuccess) e = cudaMemcpy(b->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(b->d_status, 0, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&b->d_items, count * sizeof(BatchItem));
+  if (e == cudaSuccess) e = cudaMalloc(&b->d_items, count * sizeof(SplitItem));
+  if (e == cudaSuccess) e = build_units(b);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
   for (int l = 0; l < kLanes && e == cudaSuccess; ++l) {
     e = cudaStreamCreateWithFlags(&b->lane[l], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_lane[l], cudaEventDisableTiming);
   }
-  b->sub.assign(count, nullptr);
-  b->off_sub.assign(count, 0);
   if (e != cudaSuccess) {
     fftenkf_batch_destroy(b);
     return bfail(FFTENKF_ENOMEM, "batched plan allocation failed");
-  }
-  // analyses large enough to fill the GPU through their own passes get a plan each; a shape
-  // the single-analysis plan does not take stays in the batched passes
-  for (int i = 0; i < count; ++i) {
-    if ((long long)dims[i].ny * dims[i].nx < kBigPoints) continue;
-    fftenkf_dims d = dims[i];
-    const uint8_t observed = 1;
-    fftenkf_plan sp = nullptr;
-    if (fftenkf_plan_create(&sp, &d, &observed) == FFTENKF_OK) b->sub[i] = sp;
-  }
-  set_last_error("");
-  // workspace layout, item shapes and twiddle pointers
-  size_t off = 0;
-  b->off_mean.resize(count);
-  b->off_A.resize(count);
-  b->off_W.resize(count);
-  b->off_chat.resize(count);
-  b->off_gain.resize(count);
-  for (int i = 0; i < count; ++i) {
-    BatchItem& it = b->items[i];
-    memset(&it, 0, sizeof(it));
-    it.ny = dims[i].ny;
-    it.nx = dims[i].nx;
-    it.L = it.nx / 2;
-    it.N = dims[i].n_members;
-    const size_t G = (size_t)it.ny * it.nx, line = (size_t)it.L * it.ny * sizeof(float2);
-    const size_t tab = (size_t)(it.L + 1) * it.ny * sizeof(float);
-    it.twL = b->d_tw + off_stage[0][it.L];
-    it.twL_alt = b->d_tw + off_stage[1][it.L];
-    it.twY = b->d_tw + off_stage[0][it.ny];
-    it.twY_alt = b->d_tw + off_stage[1][it.ny];
-    it.twX = b->d_tw + off_x[it.nx];
-    if (b->sub[i]) {   // the plan's workspace instead of the batched regions
-      size_t sb = 0;
-      fftenkf_workspace_size(b->sub[i], &sb);
-      b->off_sub[i] = off; off = rup(off + sb, 256);
-      b->off_mean[i] = b->off_A[i] = b->off_W[i] = b->off_chat[i] = b->off_gain[i] = b->off_sub[i];
-      continue;
-    }
-    b->off_mean[i] = off; off = rup(off + G * sizeof(float), 256);
-    b->off_A[i] = off;    off = rup(off + it.N * line, 256);
-    b->off_W[i] = off;    off = rup(off + it.N * line, 256);
-    b->off_chat[i] = off; off = rup(off + tab, 256);
-    b->off_gain[i] = off; off = rup(off + tab, 256);
-  }
-  b->ws_bytes = off;
-  for (int pass = 0; pass < kBPassCount; ++pass) {
-    fftenkf_status st = build_pass(b, pass, 256, 0);
-    if (st != FFTENKF_OK) {
-      fftenkf_batch_destroy(b);
-      return st;
-    }
   }
   *out = b;
   return FFTENKF_OK;
@@ -298,15 +243,12 @@ extern "C" fftenkf_status fftenkf_batch_destroy(fftenkf_batch b) {
   if (!b) return FFTENKF_OK;
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->cap) cudaStreamDestroy(b->cap);
-  for (fftenkf_plan sp : b->sub)
-    if (sp) fftenkf_plan_destroy(sp);
   for (int l = 0; l < kLanes; ++l) {
     if (b->lane[l]) cudaStreamDestroy(b->lane[l]);
     if (b->ev_lane[l]) cudaEventDestroy(b->ev_lane[l]);
   }
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-  for (int p = 0; p < kBPassCount; ++p)
-    if (b->d_units[p]) cudaFree(b->d_units[p]);
+  if (b->d_units) cudaFree(b->d_units);
   if (b->d_items) cudaFree(b->d_items);
   if (b->d_tw) cudaFree(b->d_tw);
   if (b->d_status) cudaFree(b->d_status);
@@ -323,26 +265,22 @@ extern "C" fftenkf_status fftenkf_batch_workspace_size(fftenkf_batch b, size_t* 
 
 static fftenkf_status bind(fftenkf_batch b, void* const* ens, const float* const* data, const void* const* pert,
                            const double* const* rhat, char* ws) {
-  bool changed = (ws != b->bound_ws);
   for (int i = 0; i < b->count; ++i) {
     if (!ens[i] || !data[i] || !pert[i] || !rhat[i]) return bfail(FFTENKF_EINVAL, "null item pointer");
     if (((uintptr_t)ens[i] | (uintptr_t)data[i] | (uintptr_t)pert[i] | (uintptr_t)rhat[i]) % 16)
       return bfail(FFTENKF_EINVAL, "item pointers must be 16-byte aligned");
-    BatchItem& it = b->items[i];
-    const bool moved = it.ens != ens[i] || it.data != data[i] || it.pert != pert[i] || it.rhat != rhat[i];
-    changed |= moved;
-    if (b->sub[i] && moved) b->sub_dirty = true;   // its kernels take the pointers by value
+  }
+  bool changed = (ws != b->bound_ws);
+  for (int i = 0; i < b->count; ++i) {
+    SplitItem& it = b->items[i];
+    changed |= it.ens != ens[i] || it.data != data[i] || it.pert != pert[i] || it.rhat != rhat[i];
     it.ens = ens[i];
     it.data = data[i];
     it.pert = pert[i];
     it.rhat = rhat[i];
-    it.mean = reinterpret_cast<float*>(ws + b->off_mean[i]);
     it.A = reinterpret_cast<float2*>(ws + b->off_A[i]);
     it.W = reinterpret_cast<float2*>(ws + b->off_W[i]);
-    it.chat = reinterpret_cast<float*>(ws + b->off_chat[i]);
-    it.gain = reinterpret_cast<float*>(ws + b->off_gain[i]);
   }
-  if (ws != b->bound_ws) b->sub_dirty = true;
   b->bound_ws = ws;
   b->items_dirty |= changed;
   return FFTENKF_OK;
@@ -376,13 +314,9 @@ extern "C" fftenkf_status fftenkf_analyze_batched(fftenkf_batch b, void* const* 
   cudaError_t e = cudaSuccess;
   if (b->items_dirty) {
     // pageable copy: the runtime stages the host table before returning, ordered on s
-    e = cudaMemcpyAsync(b->d_items, b->items.data(), b->count * sizeof(BatchItem), cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(b->d_items, b->items.data(), b->count * sizeof(SplitItem), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("item table: ") + cudaGetErrorString(e));
     b->items_dirty = false;
-  }
-  if (b->exec && b->sub_dirty) {
-    cudaGraphExecDestroy(b->exec);
-    b->exec = nullptr;
   }
   if (!b->exec) {
     cudaGraph_t g = nullptr;
@@ -390,7 +324,7 @@ extern "C" fftenkf_status fftenkf_analyze_batched(fftenkf_batch b, void* const* 
     fftenkf_status rs = FFTENKF_OK;
     std::string rmsg;
     if (e == cudaSuccess) {
-      rs = run_all(b, ensembles, data, perturbations, rhat, ws, b->cap);
+      rs = run_all(b, b->cap);
       if (rs != FFTENKF_OK) rmsg = fftenkf_last_error();
       e = cudaStreamEndCapture(b->cap, &g);
     }
@@ -404,16 +338,14 @@ extern "C" fftenkf_status fftenkf_analyze_batched(fftenkf_batch b, void* const* 
       b->exec = nullptr;
       return bfail(FFTENKF_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
     }
-    b->sub_dirty = false;
   }
   e = cudaGraphLaunch(b->exec, s);
   if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("graph launch: ") + cudaGetErrorString(e));
   return FFTENKF_OK;
 }
 
-// Time every (CTA size, schedule) candidate of every pass on zero-filled
-// scratch inputs of the batch's shapes and keep the fastest.  Allocates the
-// scratch inputs (one ensemble's worth per item) for the duration of the call.
+// Time the CTA sizes of every stage on zero-filled scratch inputs of the batch's shapes and keep the
+// fastest.  Allocates the scratch inputs (one ensemble's worth per item) for the duration of the call.
 extern "C" fftenkf_status fftenkf_batch_autotune(fftenkf_batch b, void* workspace, void* stream, double* best_ms) {
   set_last_error("");
   if (!b) return bfail(FFTENKF_EINVAL, "null argument");
@@ -425,12 +357,12 @@ extern "C" fftenkf_status fftenkf_batch_autotune(fftenkf_batch b, void* workspac
   size_t bytes = 0;
   std::vector<size_t> oe(b->count), od(b->count), op(b->count), orh(b->count);
   for (int i = 0; i < b->count; ++i) {
-    const BatchItem& it = b->items[i];
-    const size_t G = (size_t)it.ny * it.nx;
-    oe[i] = bytes; bytes = rup(bytes + it.N * G * es, 256);
+    const fftenkf_dims& d = b->dims[i];
+    const size_t G = (size_t)d.ny * d.nx;
+    oe[i] = bytes; bytes = rup(bytes + d.n_members * G * es, 256);
     od[i] = bytes; bytes = rup(bytes + G * 4, 256);
-    op[i] = bytes; bytes = rup(bytes + it.N * G * es, 256);
-    orh[i] = bytes; bytes = rup(bytes + (size_t)it.ny * (it.L + 1) * 8, 256);
+    op[i] = bytes; bytes = rup(bytes + d.n_members * G * es, 256);
+    orh[i] = bytes; bytes = rup(bytes + (size_t)d.ny * (d.nx / 2 + 1) * 8, 256);
   }
   char* scratch = nullptr;
   if (cudaMalloc(&scratch, bytes) != cudaSuccess) return bfail(FFTENKF_ENOMEM, "autotune scratch allocation failed");
@@ -444,60 +376,62 @@ extern "C" fftenkf_status fftenkf_batch_autotune(fftenkf_batch b, void* workspac
     pert[i] = scratch + op[i];
     rh[i] = reinterpret_cast<const double*>(scratch + orh[i]);
   }
-  std::vector<BatchItem> saved = b->items;
+  std::vector<SplitItem> saved = b->items;
   char* saved_ws = b->bound_ws;
   bind(b, ens.data(), dat.data(), pert.data(), rh.data(), ws);
-  cudaMemcpyAsync(b->d_items, b->items.data(), b->count * sizeof(BatchItem), cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(b->d_items, b->items.data(), b->count * sizeof(SplitItem), cudaMemcpyHostToDevice, s);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   double total = 0.0;
-  for (int pass = 0; pass < kBPassCount && st == FFTENKF_OK; ++pass) {
+  cudaError_t e = cudaSuccess;
+  for (int stage = 0; stage < kStages && e == cudaSuccess; ++stage) {
     float best = 1e30f;
-    int bbt = 256, bvs = 0;
-    const int nv = (pass == kBMean || pass == kBGain) ? 1 : 2;
-    const int nb = (pass == kBGain) ? 1 : 2;
-    for (int ci = 0; ci < nb; ++ci)
-      for (int vs = 0; vs < nv; ++vs) {
-        if (build_pass(b, pass, kCandBt[ci], vs) != FFTENKF_OK) continue;
-        const BatchParams p = pass_params(b, pass);
-        float ms = 0.f;
-        for (int rep = 0; rep < 3; ++rep) {   // first repetition warms up
-          cudaEventRecord(e0, s);
-          launch_batch_pass(pass, p, b->bt[pass], b->smem[pass], b->grid[pass], s);
-          cudaEventRecord(e1, s);
-          cudaEventSynchronize(e1);
-          float t = 0.f;
-          cudaEventElapsedTime(&t, e0, e1);
-          if (rep) ms += t;
-        }
-        if (ms < best) {
-          best = ms;
-          bbt = kCandBt[ci];
-          bvs = vs;
-        }
+    int keep = kCandBt[0];
+    for (int bt : kCandBt) {
+      b->bt[stage] = bt;
+      float ms = 0.f;
+      for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {   // first repetition warms up
+        cudaEventRecord(e0, s);
+        for (const Chunk& c : b->chunks)
+          if (e == cudaSuccess) e = run_stage(b, c, stage, s);
+        cudaEventRecord(e1, s);
+        cudaEventSynchronize(e1);
+        float t = 0.f;
+        cudaEventElapsedTime(&t, e0, e1);
+        if (rep) ms += t;
       }
-    st = build_pass(b, pass, bbt, bvs);
+      if (ms < best) {
+        best = ms;
+        keep = bt;
+      }
+    }
+    b->bt[stage] = keep;
     total += best / 2.0;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  cudaError_t e = cudaStreamSynchronize(s);
+  const cudaError_t se = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = se;
   cudaMemset(b->d_status, 0, sizeof(int));
   cudaFree(scratch);
   b->items = saved;
   b->bound_ws = saved_ws;
   b->items_dirty = true;
+  if (b->exec) {
+    cudaGraphExecDestroy(b->exec);
+    b->exec = nullptr;
+  }
   if (best_ms) *best_ms = total;
   if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("autotune: ") + cudaGetErrorString(e));
-  return st;
+  return FFTENKF_OK;
 }
 
 extern "C" fftenkf_status fftenkf_batch_schedule(fftenkf_batch b, int* cta_threads, int* sched, int n) {
   if (!b || !cta_threads || !sched) return bfail(FFTENKF_EINVAL, "null argument");
-  for (int p = 0; p < kBPassCount && p < n; ++p) {
-    cta_threads[p] = b->bt[p];
-    sched[p] = b->vsel[p];
+  for (int p = 0; p < kBatchPasses && p < n; ++p) {
+    cta_threads[p] = b->bt[stage_of(p)];
+    sched[p] = 0;   // one line plan per length
   }
   return FFTENKF_OK;
 }
@@ -510,13 +444,6 @@ extern "C" fftenkf_status fftenkf_batch_last_device_status(fftenkf_batch b, void
   e = cudaMemcpy(&word, b->d_status, sizeof(int), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemset(b->d_status, 0, sizeof(int));
   if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("status word: ") + cudaGetErrorString(e));
-  fftenkf_status worst = FFTENKF_OK;
-  for (fftenkf_plan sp : b->sub) {   // the analyses on their own plans
-    if (!sp) continue;
-    const fftenkf_status st = fftenkf_last_device_status(sp, stream);
-    if (st != FFTENKF_OK && worst == FFTENKF_OK) worst = st;
-  }
   if (word & kStatusNonFinite) return bfail(FFTENKF_ENONFINITE, "non-finite spectral covariance");
-  if (worst != FFTENKF_OK) return bfail(worst, "an analysis on its own plan: " + std::string(fftenkf_last_error()));
   return FFTENKF_OK;
 }

@@ -19,17 +19,6 @@
 
 namespace fftenkf {
 
-// (hi + lo) / n for an unevaluated sum hi + lo (an error-free accumulation) and an
-// integer n: q = hi inv_n, corrected by the remainder hi - q n (exact with an FMA,
-// since it is a small multiple of ulp(q)) plus lo.  The result is within one unit of
-// the last place of the exact quotient and equals it whenever that quotient is a
-// float (n equal members give their own value back).  inv_n = 1/n rounded.
-__device__ __forceinline__ float pair_div(float hi, float lo, float n, float inv_n) {
-  const float q = hi * inv_n;
-  const float r = fmaf(-q, n, hi) + lo;
-  return fmaf(r, inv_n, q);
-}
-
 constexpr int kMaxBlocks = 16;
 constexpr int kMaxObs = 4;
 
@@ -41,17 +30,7 @@ enum Storage { kF32 = 0, kBF16 = 1 };
 // Status bits written by kernels (OR-ed into the plan's device word).
 enum DeviceStatusBits { kStatusNonFinite = 1, kStatusTimeout = 2 };
 
-__device__ __forceinline__ float2 load2(const void* base, size_t idx, int storage) {
-  // two consecutive elements idx, idx+1 (idx even)
-  if (storage == kBF16) {
-    const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(
-        reinterpret_cast<const __nv_bfloat16*>(base) + idx);
-    return __bfloat1622float2(b);
-  }
-  return *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + idx);
-}
-
-// the same with the storage type fixed at compile time
+// two consecutive elements idx, idx+1 (idx even)
 template <int ST>
 __device__ __forceinline__ float2 load2(const void* base, size_t idx) {
   if constexpr (ST == kBF16) {
@@ -64,15 +43,6 @@ template <int ST>
 __device__ __forceinline__ void store2(void* base, size_t idx, float2 v) {
   if constexpr (ST == kBF16) {
     *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(base) + idx) = __float22bfloat162_rn(v);
-  } else {
-    *reinterpret_cast<float2*>(reinterpret_cast<float*>(base) + idx) = v;
-  }
-}
-
-__device__ __forceinline__ void store2(void* base, size_t idx, float2 v, int storage) {
-  if (storage == kBF16) {
-    *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(base) + idx) =
-        __float22bfloat162_rn(v);
   } else {
     *reinterpret_cast<float2*>(reinterpret_cast<float*>(base) + idx) = v;
   }
@@ -216,6 +186,7 @@ struct SplitParams {
   int innovations;        // forward rows: 0, kInnovation or kInnovationDrawn
   const float2 *twL, *twX, *twY;   // tables of split_row_V(L), plan_V(ny, split_col_sel)
   int R;                  // rows per tile (set by split_row_shape)
+  int threads;            // batched: threads of a CTA (0 = default)
   int groups;             // thread groups of the column pass (set by split_col_shape)
   int acc_bytes;          // shared memory of its sums
   float* chat;            // columns: covariance tables wanted instead of the update, in the col_stats layout
@@ -238,7 +209,8 @@ __host__ __device__ constexpr int split_col_sel(int ny, bool cross) {
 bool split_rows_supported(int L);
 bool split_cols_supported(int ny, int n_obs, int M);
 int split_row_tile(int L);                                    // rows per tile
-int split_col_groups(int ny, int n_obs, int M, int N);        // thread groups of one column's CTA
+// thread groups of one column's CTA (threads: limit of a batched launch, 0 = default)
+int split_col_groups(int ny, int n_obs, int M, int N, int threads = 0);
 cudaError_t launch_row_split(SplitParams p, cudaStream_t s);
 cudaError_t launch_col_split(SplitParams p, cudaStream_t s);
 cudaError_t launch_row_inv_split(SplitParams p, cudaStream_t s);

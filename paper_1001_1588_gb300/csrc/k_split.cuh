@@ -454,7 +454,8 @@ template <typename K>
 inline cudaError_t launch_rows_split(K kern, int L, int V, SplitParams p, int units, cudaStream_t st) {
   const int T = L / V;
   p.R = split_row_tile(L);
-  int lpc = 256 / T;
+  int lpc = (p.threads ? p.threads : 256) / T;
+  if (lpc < 1) lpc = 1;
   if (lpc > p.R) lpc = p.R;
   const size_t smem = (size_t)p.R * row_pitch(L) * sizeof(float2);
   int per_sm = 0;

@@ -221,8 +221,7 @@ int sm_count();
 
 struct GainParams {
   int ny, L, n_obs, n_un;
-  const float* chat_t;    // stats kernel output (transposed, float), or null
-  const double* spec;     // caller spectrum (natural layout, double), or null
+  const double* spec;     // caller spectrum (natural layout, double)
   const double* rhat;     // [n_obs][ny][L+1]
   float* goo;
   float2* gjo;

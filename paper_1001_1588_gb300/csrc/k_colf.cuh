@@ -27,6 +27,7 @@
 // another.
 #pragma once
 #include "common.cuh"
+#include "dd.cuh"
 #include "fft_pair.cuh"
 #include "perturb.cuh"
 #include "tma.cuh"
@@ -164,7 +165,8 @@ __device__ __forceinline__ void fused_accumulate(const cp (&v)[V], int pp, int M
 
 // Sums -> gains in place (analysis), or -> covariance tables in global memory (statistics
 // only), for the wavenumbers (t + T m, column c) of this thread.  The denominator
-// chat^(oo) + rhat is formed in FP64 and rounded once; the quotients are FP32, or FP64 where
+// chat^(oo) + rhat is formed in float pairs (dd.cuh; in FP64 the gain step took 0.97 ms of the pass at
+// 4096^2 with two observed blocks) and rounded once; the quotients are FP32, or FP64 where
 // the rounded denominator is below FLT_MIN (0 where it is exactly 0, as in the oracle).  With
 // the pivot form chat^(oo) can come out a few rounding errors below 0 where the ensemble has
 // no variance above FFT round-off; with rhat = 0 such a wavenumber keeps the gain 1 of
@@ -184,31 +186,30 @@ __device__ __forceinline__ bool fused_gains(const ColFusedParams& p, uint32_t ta
     float a[V];
     tm_ld<V>(ta + i * V, a);
     float val[V], inv[V];
-    double rr[V];
     unsigned tiny = 0;
 #pragma unroll
     for (int m = 0; m < V; ++m) {
       val[m] = a[m] * p.scale;
       ok &= isfinite(val[m]);
     }
+    const double* rh = p.rhat_t + i * tab + (size_t)c * NY + t;
     if (stats_only) {
 #pragma unroll
       for (int m = 0; m < V; ++m) p.chat[i * tab + (size_t)c * NY + t + T * m] = val[m];
     } else {
+      double rr[V];
 #pragma unroll
-      for (int m = 0; m < V; ++m) rr[m] = __ldg(p.rhat_t + i * tab + (size_t)c * NY + t + T * m);
+      for (int m = 0; m < V; ++m) rr[m] = __ldg(rh + T * m);
 #pragma unroll
       for (int m = 0; m < V; ++m) {
-        const double den = (double)val[m] + rr[m];
-        const float denf = (float)den;
-        if (denf >= 1.17549435e-38f) {
-          inv[m] = __fdividef(p.inv_G, denf);
+        float den;
+        if (denominator(val[m], rr[m], den)) {
+          inv[m] = __fdividef(p.inv_G, den);
           a[m] = val[m] * inv[m];
         } else {
           tiny |= 1u << m;
-          const double rd = (den != 0.0) ? (double)p.inv_G / den : 0.0;
           inv[m] = 0.f;
-          a[m] = (float)((double)val[m] * rd);
+          a[m] = (float)((double)val[m] * quotient_fp64(val[m], rr[m], p.inv_G));
         }
       }
       tm_st<V>(ta + i * V, a);
@@ -225,8 +226,7 @@ __device__ __forceinline__ bool fused_gains(const ColFusedParams& p, uint32_t ta
         if (stats_only) {
           xout[(size_t)(i * p.n_un + u) * tab + (size_t)c * NY + t + T * m] = make_float2(xr, xi);
         } else if (tiny & (1u << m)) {
-          const double den = (double)val[m] + rr[m];
-          const double rd = (den != 0.0) ? (double)p.inv_G / den : 0.0;
+          const double rd = quotient_fp64(val[m], __ldg(rh + T * m), p.inv_G);
           x[2 * m] = (float)((double)xr * rd);
           x[2 * m + 1] = (float)((double)xi * rd);
         } else {

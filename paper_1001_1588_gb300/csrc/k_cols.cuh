@@ -18,6 +18,7 @@
 // transform for every target block and writes the increment's row spectra.
 #pragma once
 #include "common.cuh"
+#include "dd.cuh"
 #include "perturb.cuh"
 #include "tma.cuh"
 
@@ -214,14 +215,13 @@ __global__ void __launch_bounds__((NY / V > 256) ? 512 : 256, 1) col_stats_kerne
             if (p.chat) p.chat[i * tab + at] = val;
             if (p.rhat_t) {
               // eq. (spectral-multi-enkf): G = chat / (chat^(oo) + rhat).  The sum is formed in
-              // FP64 (where chat << rhat it keeps chat's digits), then rounded once; the
+              // float pairs (where chat << rhat it keeps chat's digits), then rounded once; the
               // quotients are FP32; a sum below FLT_MIN takes the FP64 path (gains_fp64).
-              const double den = (double)val + rr[e];
-              const float denf = (float)den;
+              float denf;
+              const bool tiny = !denominator(val, rr[e], denf);
               const float inv = __fdividef(p.inv_G, denf);
-              const bool tiny = !(denf >= 1.17549435e-38f);
               if (tiny) {
-                bad |= !gains_fp64(p.goo, p.gjo, xout, xacc + ky, NY, i, p.n_un, at, tab, den, val, p.inv_G, p.scale);
+                bad |= !gains_fp64(p.goo, p.gjo, xout, xacc + ky, NY, i, p.n_un, at, tab, (double)val + rr[e], val, p.inv_G, p.scale);
               } else {
                 p.goo[i * tab + at] = val * inv;
                 for (int u = 0; u < p.n_un; ++u) {

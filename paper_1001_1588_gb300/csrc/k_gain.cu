@@ -1,5 +1,5 @@
-// Gain tables of eq. (spectral-enkf) / eq. (spectral-multi-enkf), computed in
-// FP64 per wavenumber, and the transpose of the covariance tables to the
+// Gain tables of eq. (spectral-enkf) / eq. (spectral-multi-enkf) from a caller's
+// spectrum, in float pairs per wavenumber (dd.cuh), and the transpose of the covariance tables to the
 // boundary's [k_y][k_x] layout.
 //
 //   G^(oo) = chat^(oo) / (chat^(oo) + rhat_o),  G^(jo) = chat^(jo) / (chat^(oo) + rhat_o)
@@ -12,23 +12,11 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "dd.cuh"
 
 namespace fftenkf {
 
 constexpr int TB = 32;
-
-// 1/x in FP64 for normal x > 0: the hardware's approximate reciprocal refined
-// by two steps of the Newton-Raphson iteration for f(y) = 1/y - x
-// (e <- 1 - x y, y <- y + y e), each of which doubles the correct bits.
-// Subnormal or zero x are handled by the caller.
-__device__ __forceinline__ double recip64(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
-}
 
 // load a [ny][L+1] double tile (rows ky0.., cols c0..) into s[ky][c]
 __device__ __forceinline__ void load_tile(double (*s)[TB + 1], const double* __restrict__ src, int ny, int L1,
@@ -49,53 +37,41 @@ __global__ void __launch_bounds__(256) gain_kernel(const GainParams p) {
   const size_t K = (size_t)p.ny * L1;   // doubles per real table (natural layout)
   const size_t tab = (size_t)L1 * p.ny;  // elements per transposed table
   load_tile(rs, p.rhat + i * K, p.ny, L1, ky0, c0, 1, 0);
-  if (p.spec) load_tile(ca, p.spec + i * K, p.ny, L1, ky0, c0, 1, 0);
+  load_tile(ca, p.spec + i * K, p.ny, L1, ky0, c0, 1, 0);
   __syncthreads();
   // thread (x -> ky offset, y -> column offset): coalesced along k_y on output
   const int ky = ky0 + threadIdx.x;
-  double inv[TB / 8];
   bool bad = false;
+  auto quotient = [&](int q) {   // of this thread's q-th wavenumber (entries off the grid are 0)
+    const int cl = threadIdx.y + 8 * q;
+    return SpecQuotient(ca[threadIdx.x][cl], rs[threadIdx.x][cl], p.scale);
+  };
+  const SpecQuotient inv[TB / 8] = {quotient(0), quotient(1), quotient(2), quotient(3)};
 #pragma unroll
   for (int q = 0; q < TB / 8; ++q) {
     const int cl = threadIdx.y + 8 * q;
     const int c = c0 + cl;
-    inv[q] = 0.0;
     if (c < L1 && ky < p.ny) {
-      const double a = p.spec ? ca[threadIdx.x][cl] : (double)p.chat_t[i * tab + (size_t)c * p.ny + ky];
-      bad |= !isfinite(a);
-      const double den = a + rs[threadIdx.x][cl];
-      inv[q] = (den > 1e-300) ? recip64(den) : ((den != 0.0) ? 1.0 / den : 0.0);
-      inv[q] *= (double)p.scale;
-      p.goo[i * tab + (size_t)c * p.ny + ky] = (float)(a * inv[q]);
+      const double a = ca[threadIdx.x][cl];
+      bad |= !finite_double(a);
+      p.goo[i * tab + (size_t)c * p.ny + ky] = inv[q].times(a);
     }
   }
-  const double* xspec = p.spec ? p.spec + (size_t)p.n_obs * K : nullptr;
-  const float2* xchat = reinterpret_cast<const float2*>(p.chat_t + (size_t)p.n_obs * tab);
+  const double* xspec = p.spec + (size_t)p.n_obs * K;
   for (int u = 0; u < p.n_un; ++u) {
     const int qt = i * p.n_un + u;
-    if (p.spec) {
-      __syncthreads();
-      load_tile(cre, xspec + (size_t)qt * 2 * K, p.ny, L1, ky0, c0, 2, 0);
-      load_tile(cim, xspec + (size_t)qt * 2 * K, p.ny, L1, ky0, c0, 2, 1);
-      __syncthreads();
-    }
+    __syncthreads();
+    load_tile(cre, xspec + (size_t)qt * 2 * K, p.ny, L1, ky0, c0, 2, 0);
+    load_tile(cim, xspec + (size_t)qt * 2 * K, p.ny, L1, ky0, c0, 2, 1);
+    __syncthreads();
 #pragma unroll
     for (int q = 0; q < TB / 8; ++q) {
       const int cl = threadIdx.y + 8 * q;
       const int c = c0 + cl;
       if (c < L1 && ky < p.ny) {
-        double re, im;
-        if (p.spec) {
-          re = cre[threadIdx.x][cl];
-          im = cim[threadIdx.x][cl];
-        } else {
-          const float2 v = xchat[qt * tab + (size_t)c * p.ny + ky];
-          re = v.x;
-          im = v.y;
-        }
-        bad |= !(isfinite(re) && isfinite(im));
-        const double sc = inv[q];
-        p.gjo[qt * tab + (size_t)c * p.ny + ky] = make_float2((float)(re * sc), (float)(im * sc));
+        const double re = cre[threadIdx.x][cl], im = cim[threadIdx.x][cl];
+        bad |= !(finite_double(re) && finite_double(im));
+        p.gjo[qt * tab + (size_t)c * p.ny + ky] = make_float2(inv[q].times(re), inv[q].times(im));
       }
     }
   }
@@ -145,11 +121,11 @@ __global__ void __launch_bounds__(256) chat_out_kernel(const float* __restrict__
     if (ky < ny && c < L1) {
       const float2 v = tile[threadIdx.x][yy];
       if (is_auto) {
-        out[q * K + (size_t)ky * L1 + c] = v.x;
+        out[q * K + (size_t)ky * L1 + c] = to_double(v.x);
       } else {
         double* o = out + map.n_auto * K + (size_t)(q - map.n_auto) * 2 * K + ((size_t)ky * L1 + c) * 2;
-        o[0] = v.x;
-        o[1] = v.y;
+        o[0] = to_double(v.x);
+        o[1] = to_double(v.y);
       }
     }
   }
@@ -211,7 +187,7 @@ __global__ void __launch_bounds__(256) rhat_transpose_kernel(const double* __res
     if (c < L1 && ky < ny) {
       const double r = tile[threadIdx.x][cc];
       dst[(size_t)c * ny + ky] = r;
-      if (amp) amp[blockIdx.z * K + (size_t)c * ny + ky] = sqrt_G * sqrtf((float)r);
+      if (amp) amp[blockIdx.z * K + (size_t)c * ny + ky] = sqrt_G * sqrtf(to_float(r));
     }
   }
 }
@@ -223,9 +199,45 @@ cudaError_t launch_rhat_transpose(const double* rhat, double* rhat_t, int n, int
   return cudaGetLastError();
 }
 
-// One thread per wavenumber (column-major index at = k_x ny + k_y).  The bracket
-// A = chat_OO + diag(rhat) is inverted in FP64: A^-1 when det A > 1e-6 a11 a22, the
-// pseudo-inverse A / tr(A)^2 of a rank-1 bracket otherwise, 0 where tr(A) = 0; it is
+// g A^-1 of the bracket A = [[a0 + r0, conj b], [b, a1 + r1]] in FP64: A^-1 when det A > 1e-6 a11 a22, the
+// pseudo-inverse A / tr(A)^2 of a rank-1 bracket otherwise, 0 where tr(A) = 0; rounded to float.
+struct Bracket {
+  float s00, s11;
+  float2 s01;
+};
+static __device__ __noinline__ Bracket bracket_fp64(float a0, float a1, float2 b, double r0, double r1, float g) {
+  const double a = (double)a0 + r0, d = (double)a1 + r1;
+  const double br = b.x, bi = b.y;
+  const double det = a * d - (br * br + bi * bi);
+  const double tr = a + d;
+  double f = 0.0, q00 = 0.0, q11 = 0.0, q01r = 0.0, q01i = 0.0;   // A^-1 = f [[q00, q01], [conj q01, q11]]
+  if (det > 1e-6 * a * d) {
+    f = (double)g / det;
+    q00 = d; q11 = a; q01r = -br; q01i = bi;      // [[d, -conj b], [-b, a]] / det
+  } else if (tr > 0.0) {
+    f = (double)g / (tr * tr);
+    q00 = a; q11 = d; q01r = br; q01i = -bi;      // [[a, conj b], [b, d]] / tr^2
+  }
+  return {(float)(f * q00), (float)(f * q11), make_float2((float)(f * q01r), (float)(f * q01i))};
+}
+// The same in float pairs (48 bits; the determinant keeps at least 28 of them where it is used, since
+// it is above 1e-6 of the product of the diagonal).
+__device__ __forceinline__ Bracket bracket(float a0, float a1, float2 b, double r0, double r1, float g) {
+  fpair p0, p1;
+  const bool in = split_double(r0, p0) & split_double(r1, p1);
+  const fpair a = pair_add({a0, 0.f}, p0), d = pair_add({a1, 0.f}, p1);
+  const fpair ad = pair_mul(a, d);
+  const fpair bb = pair_add(pair_mul({b.x, 0.f}, {b.x, 0.f}), pair_mul({b.y, 0.f}, {b.y, 0.f}));
+  const fpair det = pair_add(ad, {-bb.h, -bb.l});
+  if (!in || !(det.h > 2e-6f * ad.h) || !well_inside(det.h) || !well_inside(a.h) || !well_inside(d.h))
+    return bracket_fp64(a0, a1, b, r0, r1, g);   // (nearly) singular, or out of the pairs' range
+  const fpair f = pair_recip(det);
+  return {pair_product(f, d, g), pair_product(f, a, g),
+          make_float2(pair_product(f, {-b.x, 0.f}, g), pair_product(f, {b.y, 0.f}, g))};
+}
+
+// One thread per wavenumber (column-major index at = k_x ny + k_y).  The bracket A = chat_OO +
+// diag(rhat) is inverted (bracket above; in FP64 the kernel took 465 us at 4096^2 with three blocks),
 // scaled by 1/(ny nx) and rounded to float, and K_r = chat_{r,O} A^-1 is formed in FP32.
 __global__ void __launch_bounds__(256) coupled_gain_kernel(const CoupledGainParams p) {
   const size_t tab = (size_t)(p.L + 1) * p.ny;
@@ -237,26 +249,15 @@ __global__ void __launch_bounds__(256) coupled_gain_kernel(const CoupledGainPara
     const float2 b10 = (p.n_obs == 2) ? cx[at] : make_float2(0.f, 0.f);   // chat^(o1 o0)
     float s00 = 0.f, s11 = 0.f;
     float2 s01 = make_float2(0.f, 0.f);
-    const double g = (double)p.inv_G;
     if (p.n_obs == 1) {
-      const double a = (double)a0 + p.rhat_t[at];
-      s00 = (a != 0.0) ? (float)(g / a) : 0.f;
+      const double r = p.rhat_t[at];
+      float den;
+      s00 = denominator(a0, r, den) ? __fdiv_rn(p.inv_G, den) : (float)quotient_fp64(a0, r, p.inv_G);
     } else {
-      const double a = (double)a0 + p.rhat_t[at], d = (double)a1 + p.rhat_t[tab + at];
-      const double br = b10.x, bi = b10.y;
-      const double det = a * d - (br * br + bi * bi);
-      const double tr = a + d;
-      double f = 0.0, q00 = 0.0, q11 = 0.0, q01r = 0.0, q01i = 0.0;   // A^-1 = f [[q00, q01], [conj q01, q11]]
-      if (det > 1e-6 * a * d) {
-        f = g / det;
-        q00 = d; q11 = a; q01r = -br; q01i = bi;      // [[d, -conj b10], [-b10, a]] / det
-      } else if (tr > 0.0) {
-        f = g / (tr * tr);
-        q00 = a; q11 = d; q01r = br; q01i = -bi;      // [[a, conj b10], [b10, d]] / tr^2
-      }
-      s00 = (float)(f * q00);
-      s11 = (float)(f * q11);
-      s01 = make_float2((float)(f * q01r), (float)(f * q01i));
+      const Bracket k = bracket(a0, a1, b10, p.rhat_t[at], p.rhat_t[tab + at], p.inv_G);
+      s00 = k.s00;
+      s11 = k.s11;
+      s01 = k.s01;
     }
     const float2 s10 = make_float2(s01.x, -s01.y);
     bad |= !(isfinite(s00) && isfinite(s11) && isfinite(s01.x) && isfinite(s01.y));

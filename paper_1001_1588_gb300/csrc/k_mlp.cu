@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "dd.cuh"
 #include "launch.cuh"
 
 namespace fftenkf {
@@ -62,7 +63,7 @@ __global__ void __launch_bounds__(256) mlp_max_kernel(const MlpBinParams p) {
   stream_order_wait();
   float mx = 0.f;
 #pragma unroll 4
-  for (int i = blockIdx.x * 256 + threadIdx.x; i < p.bins.K1; i += gridDim.x * 256) mx = fmaxf(mx, (float)c[i]);
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < p.bins.K1; i += gridDim.x * 256) mx = fmaxf(mx, to_float(c[i]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0) red8[threadIdx.x >> 5] = mx;
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(256) mlp_binsum_kernel(const MlpBinParams p) {
   const double* c = p.chat + (size_t)blockIdx.y * p.bins.K1;
   float v[E];
 #pragma unroll
-  for (int e = 0; e < E; ++e) v[e] = at[e] != ~0u ? (float)c[at[e]] : 0.f;
+  for (int e = 0; e < E; ++e) v[e] = at[e] != ~0u ? to_float(c[at[e]]) : 0.f;
   const float inv = 1.f / cmax_of(p.bins, blockIdx.y, &cm);
   float acc = 0.f;
 #pragma unroll
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(256) mlp_unbin_kernel(const MlpUnbinParams p) 
       const float fr = pos - b;
       v = p.out_log[b] + fr * (p.out_log[b + 1] - p.out_log[b]);
     }
-    p.chat_out[i] = (double)expf(v);
+    p.chat_out[i] = to_double(expf(v));
   }
 }
 

@@ -15,6 +15,7 @@
 // of units).
 #pragma once
 #include "common.cuh"
+#include "dd.cuh"
 #include "k_cols.cuh"
 #include "k_rows.cuh"
 #include "launch.cuh"
@@ -191,21 +192,11 @@ __global__ void __launch_bounds__(256, 2) row_inv_split_kernel(const __grid_cons
 }
 
 // ----------------------------------------------------------------- columns
-// 1/x in FP64 for normal x > 0: the hardware's approximate reciprocal refined by two Newton-Raphson
-// steps for f(y) = 1/y - x, each of which doubles the correct bits.
-__device__ __forceinline__ double recip64_s(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
-}
-
 // Sums over the groups -> gains (in the first group's region), or covariance tables when the spectrum
 // alone is wanted, or gains of a caller's spectrum; one thread per wavenumber.  The denominator is
-// formed in FP64 and rounded once, the quotients are FP32, or FP64 where the rounded denominator is below
-// FLT_MIN (0 where it is exactly 0); with a caller's spectrum everything is FP64.  False if a value is not finite.
+// formed in float pairs (dd.cuh) and rounded once, the quotients are FP32, or FP64 where the rounded
+// denominator is below FLT_MIN (0 where it is exactly 0); with a caller's spectrum the quotients are
+// formed in pairs too.  False if a value is not finite.
 template <int NY>
 __device__ __forceinline__ bool split_gains(const SplitParams& p, const SplitItem& it, float* acc, int G, int nf, int c) {
   const size_t tab = (size_t)(p.L + 1) * NY;
@@ -219,14 +210,13 @@ __device__ __forceinline__ bool split_gains(const SplitParams& p, const SplitIte
       if (p.spec) {
         const size_t at = (size_t)ky * (p.L + 1) + c;
         const double a = p.spec[(size_t)i * tab + at];
-        ok &= (bool)isfinite(a);
-        const double den = a + rr;
-        const double inv = ((den > 1e-300) ? recip64_s(den) : ((den != 0.0) ? 1.0 / den : 0.0)) * (double)p.inv_G;
-        acc[i * NY + ky] = (float)(a * inv);
-        for (int q = 0; q < n_un; ++q) {
-          const double* s = p.spec + (size_t)p.n_obs * tab + 2 * ((size_t)(i * n_un + q) * tab + at);
-          ok &= isfinite(s[0]) && isfinite(s[1]);
-          x0[(size_t)q * NY] = make_float2((float)(s[0] * inv), (float)(s[1] * inv));
+        ok &= finite_double(a);
+        const SpecQuotient q(a, rr, p.inv_G);
+        acc[i * NY + ky] = q.times(a);
+        for (int u = 0; u < n_un; ++u) {
+          const double* s = p.spec + (size_t)p.n_obs * tab + 2 * ((size_t)(i * n_un + u) * tab + at);
+          ok &= finite_double(s[0]) && finite_double(s[1]);
+          x0[(size_t)u * NY] = make_float2(q.times(s[0]), q.times(s[1]));
         }
         continue;
       }
@@ -234,11 +224,10 @@ __device__ __forceinline__ bool split_gains(const SplitParams& p, const SplitIte
       for (int g = 0; g < G; ++g) val += acc[(size_t)g * nf * NY + i * NY + ky];
       val *= scale;
       ok &= (bool)isfinite(val);
-      const double den = (double)val + rr;
-      const float denf = (float)den;
-      const bool tiny = !(denf >= 1.17549435e-38f);
+      float denf;
+      const bool tiny = !denominator(val, rr, denf);
       const float inv = __fdividef(p.inv_G, denf);
-      const double rd = (tiny && den != 0.0) ? (double)p.inv_G / den : 0.0;
+      const double rd = (tiny && !p.chat) ? quotient_fp64(val, rr, p.inv_G) : 0.0;
       if (p.chat) p.chat[i * tab + (size_t)c * NY + ky] = val;
       else acc[i * NY + ky] = tiny ? (float)((double)val * rd) : val * inv;
       for (int q = 0; q < n_un; ++q) {
@@ -272,15 +261,15 @@ __device__ __forceinline__ void add_drawn(float2 (&v)[V], unsigned long long see
       const uint4 w4 = philox4x32_10(make_uint4((uint32_t)(t + T * m), (uint32_t)c, (uint32_t)stream, 0u),
                                      (uint32_t)seed, (uint32_t)(seed >> 32));
       const float2 zl = box_muller(w4.x, w4.y), zh = box_muller(w4.z, w4.w);
-      const float al = h * sqrt_G * sqrtf((float)rh[(size_t)(t + T * m) * ys]);
-      const float ah = h * sqrt_G * sqrtf((float)rh[(size_t)(t + T * (m + V / 2)) * ys]);
+      const float al = h * sqrt_G * sqrtf(to_float(rh[(size_t)(t + T * m) * ys]));
+      const float ah = h * sqrt_G * sqrtf(to_float(rh[(size_t)(t + T * (m + V / 2)) * ys]));
       v[m] = make_float2(fmaf(al, zl.x, v[m].x), fmaf(al, zl.y, v[m].y));
       v[m + V / 2] = make_float2(fmaf(ah, zh.x, v[m + V / 2].x), fmaf(ah, zh.y, v[m + V / 2].y));
     }
   } else {
 #pragma unroll
     for (int m = 0; m < V; ++m) {
-      const float a = sqrt_G * sqrtf((float)rh[(size_t)(t + T * m) * ys]);
+      const float a = sqrt_G * sqrtf(to_float(rh[(size_t)(t + T * m) * ys]));
       const float2 z = white_edge(seed, stream, t + T * m, c, NY);
       v[m] = make_float2(fmaf(a, z.x, v[m].x), fmaf(a, z.y, v[m].y));
     }

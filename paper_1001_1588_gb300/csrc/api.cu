@@ -64,8 +64,6 @@ struct fftenkf_plan_s {
   int obs_of_block[kMaxBlocks];
   int un_of_block[kMaxBlocks];
   float2* d_tw = nullptr;     // [L] row twiddles, [ny] column twiddles, [L+1] real-FFT twiddles
-  float4* d_tw4 = nullptr;    // paired column twiddles of the fused column pass, both schedules
-  size_t off_tw4[2] = {0, 0};
   bool fused_ok[2] = {false, false};   // the fused column pass covers the plan with schedule 0 / 1
   int* d_status = nullptr;
   cudaStream_t aux = nullptr;
@@ -222,20 +220,7 @@ extern "C" fftenkf_status fftenkf_plan_create(fftenkf_plan* plan, const fftenkf_
     return fail(FFTENKF_ENOMEM, "twiddle allocation failed");
   }
   e = cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
-  std::vector<float4> t4;
-  for (int sel = 0; sel < 2; ++sel) {
-    p->fused_ok[sel] = col_fused_supported(p->ny, p->n_obs, p->M, sel);
-    if (!p->fused_ok[sel]) continue;
-    std::vector<float2> t1;
-    host_stage_twiddles(t1, p->ny, plan_V(p->ny, sel));
-    p->off_tw4[sel] = t4.size();
-    for (const float2& w : t1) t4.push_back(make_float4(w.x, w.x, w.y, w.y));
-    t4.push_back(make_float4(0.f, 0.f, 0.f, 0.f));
-  }
-  if (e == cudaSuccess && !t4.empty()) {
-    e = cudaMalloc(&p->d_tw4, t4.size() * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_tw4, t4.data(), t4.size() * sizeof(float4), cudaMemcpyHostToDevice);
-  }
+  for (int sel = 0; sel < 2; ++sel) p->fused_ok[sel] = col_fused_supported(p->ny, p->n_obs, p->M, sel);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->aux, cudaStreamNonBlocking);
@@ -253,7 +238,6 @@ extern "C" fftenkf_status fftenkf_plan_destroy(fftenkf_plan p) {
   if (!p) return FFTENKF_OK;
   if (p->own_ws) cudaFree(p->own_ws);
   if (p->d_tw) cudaFree(p->d_tw);
-  if (p->d_tw4) cudaFree(p->d_tw4);
   if (p->d_status) cudaFree(p->d_status);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
@@ -358,7 +342,7 @@ static ColFusedParams fused_params(fftenkf_plan p, char* ws) {
   f.A = reinterpret_cast<const float2*>(ws + p->off_A);
   f.S = reinterpret_cast<float2*>(ws + p->off_A);
   f.vsel = p->sched[kPassFused] & 1;
-  f.tw = p->d_tw4 + p->off_tw4[f.vsel];
+  f.tw = p->twY(f.vsel);
   f.scale = (float)(1.0 / ((double)(p->N - 1) * (double)p->ny * (double)p->nx));
   f.inv_G = (float)(1.0 / ((double)p->ny * (double)p->nx));
   f.status = p->d_status;

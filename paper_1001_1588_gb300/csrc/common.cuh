@@ -146,7 +146,7 @@ struct ColFusedParams {
   float2* S;              // increment row spectra, field j*N+k (may alias A)
   const double* rhat_t;   // [n_obs][L+1][ny] (analysis)
   float* chat;            // statistics only: tables in the col_stats layout
-  const float4* tw;       // paired compact stage twiddles of the ny-point plan
+  const float2* tw;       // compact stage twiddles of the ny-point plan
   float scale;            // 1 / ((N-1) ny nx)
   float inv_G;            // 1 / (ny nx)
   int* status;

@@ -119,79 +119,162 @@ template <bool INV> struct Dft<4, INV> {
   }
 };
 
-// multiply by exp(-+ 2 pi i e / 8) for e = 1, 2, 3
-template <int E, bool INV>
-__device__ __forceinline__ float2 w8(float2 v) {
-  const float c = 0.70710678118654752440f;
-  if (E == 0) return v;
-  if (E == 2) return rot90<INV>(v);
-  if (E == 1) return INV ? make_float2(c * (v.x - v.y), c * (v.x + v.y))
-                         : make_float2(c * (v.x + v.y), c * (v.y - v.x));
-  // E == 3
-  return INV ? make_float2(-c * (v.x + v.y), c * (v.x - v.y))
-             : make_float2(c * (v.y - v.x), -c * (v.x + v.y));
+// The 8- and 16-point DFTs, written once for one line (complex float2) and for two at a time (fft_pair.cuh).
+// Rotations by odd multiples of pi/8 are taken as a scale times a shear (cos a (1 - i tan a)), and every scale goes
+// into the fused multiply-adds of the butterfly that follows: 144 operations for 16 points (161 with the
+// rotations as products), 52 for 8.
+struct LineOps {
+  using C = float2;
+  using S = float;
+  static __device__ __forceinline__ S re(const C& c) { return c.x; }
+  static __device__ __forceinline__ S im(const C& c) { return c.y; }
+  static __device__ __forceinline__ C mk(S r, S i) { return make_float2(r, i); }
+  static __device__ __forceinline__ S add(S a, S b) { return a + b; }
+  static __device__ __forceinline__ S sub(S a, S b) { return a - b; }
+  static __device__ __forceinline__ S fma(float k, S a, S b) { return fmaf(k, a, b); }
+};
+template <class O> __device__ __forceinline__ typename O::C c_add(typename O::C a, typename O::C b) {
+  return O::mk(O::add(O::re(a), O::re(b)), O::add(O::im(a), O::im(b)));
+}
+template <class O> __device__ __forceinline__ typename O::C c_sub(typename O::C a, typename O::C b) {
+  return O::mk(O::sub(O::re(a), O::re(b)), O::sub(O::im(a), O::im(b)));
+}
+// a + k d
+template <class O> __device__ __forceinline__ typename O::C c_fma(float k, typename O::C d, typename O::C a) {
+  return O::mk(O::fma(k, O::re(d), O::re(a)), O::fma(k, O::im(d), O::im(a)));
+}
+// a + k s d, s = -i (forward) or +i (INV)
+template <class O, bool INV>
+__device__ __forceinline__ typename O::C c_fma_rot(float k, typename O::C d, typename O::C a) {
+  return INV ? O::mk(O::fma(-k, O::im(d), O::re(a)), O::fma(k, O::re(d), O::im(a)))
+             : O::mk(O::fma(k, O::im(d), O::re(a)), O::fma(-k, O::re(d), O::im(a)));
+}
+template <class O, bool INV>
+__device__ __forceinline__ typename O::C c_add_rot(typename O::C a, typename O::C d) {
+  return INV ? O::mk(O::sub(O::re(a), O::im(d)), O::add(O::im(a), O::re(d)))
+             : O::mk(O::add(O::re(a), O::im(d)), O::sub(O::im(a), O::re(d)));
+}
+template <class O, bool INV>
+__device__ __forceinline__ typename O::C c_sub_rot(typename O::C a, typename O::C d) {
+  return c_add_rot<O, !INV>(a, d);
+}
+template <class O, bool INV>
+__device__ __forceinline__ void dft4(typename O::C& a0, typename O::C& a1, typename O::C& a2, typename O::C& a3) {
+  using C = typename O::C;
+  const C t0 = c_add<O>(a0, a2), t1 = c_sub<O>(a0, a2), t2 = c_add<O>(a1, a3), d = c_sub<O>(a1, a3);
+  a0 = c_add<O>(t0, t2);
+  a2 = c_sub<O>(t0, t2);
+  a1 = c_add_rot<O, INV>(t1, d);
+  a3 = c_sub_rot<O, INV>(t1, d);
+}
+// v exp(-+ i pi/4) sqrt(2)
+template <class O, bool INV> __device__ __forceinline__ typename O::C c_eighth(typename O::C v) {
+  return c_add_rot<O, INV>(v, v);
+}
+template <class O, bool INV>
+__device__ __forceinline__ void dft8(typename O::C* a) {
+  using C = typename O::C;
+  constexpr float c = 0.70710678118654752440f;
+  dft4<O, INV>(a[0], a[2], a[4], a[6]);
+  dft4<O, INV>(a[1], a[3], a[5], a[7]);
+  const C e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6], o0 = a[1], o1 = c_eighth<O, INV>(a[3]), o2 = a[5], v = a[7];
+  a[0] = c_add<O>(e0, o0);
+  a[4] = c_sub<O>(e0, o0);
+  a[1] = c_fma<O>(c, o1, e1);
+  a[5] = c_fma<O>(-c, o1, e1);
+  a[2] = c_add_rot<O, INV>(e2, o2);
+  a[6] = c_sub_rot<O, INV>(e2, o2);
+  // exp(-+ 3 i pi/4) v: forward c (im - re, -(re + im)), inverse c (-(re + im), re - im)
+  const typename O::S s = O::add(O::re(v), O::im(v)), d = O::sub(O::im(v), O::re(v));
+  if (INV) {
+    a[3] = O::mk(O::fma(-c, s, O::re(e3)), O::fma(-c, d, O::im(e3)));
+    a[7] = O::mk(O::fma(c, s, O::re(e3)), O::fma(c, d, O::im(e3)));
+  } else {
+    a[3] = O::mk(O::fma(c, d, O::re(e3)), O::fma(-c, s, O::im(e3)));
+    a[7] = O::mk(O::fma(-c, d, O::re(e3)), O::fma(c, s, O::im(e3)));
+  }
+}
+
+template <class O, bool INV>
+__device__ __forceinline__ void dft16(typename O::C* a) {
+  using C = typename O::C;
+  using S = typename O::S;
+  constexpr float c = 0.70710678118654752440f;     // cos(pi/4)
+  constexpr float c1 = 0.92387953251128675613f;    // cos(pi/8)
+  constexpr float tn = 0.41421356237309504880f;    // tan(pi/8)
+  constexpr float T = INV ? -tn : tn;
+  // 16 = 4 x 4: DFT4 over a[4 n1 + n2], twiddle W16^(n2 k1), DFT4 over n2
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) dft4<O, INV>(a[n2], a[4 + n2], a[8 + n2], a[12 + n2]);
+  // a[4 k1 + n2] holds y[n2][k1]
+  dft4<O, INV>(a[0], a[1], a[2], a[3]);   // k1 = 0
+  {   // k1 = 1: W16^1 y1 = c1 u1, W8 y2 = c z, W16^3 y3 = c1 u3
+    const C y0 = a[4], y1 = a[5], y2 = a[6], y3 = a[7];
+    const C u1 = O::mk(O::fma(T, O::im(y1), O::re(y1)), O::fma(-T, O::re(y1), O::im(y1)));
+    const C z = c_eighth<O, INV>(y2);
+    const C t0 = c_fma<O>(c, z, y0), t1 = c_fma<O>(-c, z, y0);
+    // forward u3 = (tan re + im, -(re - tan im)), inverse u3 = (-(im - tan re), re + tan im)
+    const S p = O::fma(tn, INV ? O::im(y3) : O::re(y3), INV ? O::re(y3) : O::im(y3));
+    const S m = O::fma(-tn, INV ? O::re(y3) : O::im(y3), INV ? O::im(y3) : O::re(y3));
+    const C s = INV ? O::mk(O::sub(O::re(u1), m), O::add(O::im(u1), p)) : O::mk(O::add(O::re(u1), p), O::sub(O::im(u1), m));
+    const C d = INV ? O::mk(O::add(O::re(u1), m), O::sub(O::im(u1), p)) : O::mk(O::sub(O::re(u1), p), O::add(O::im(u1), m));
+    a[4] = c_fma<O>(c1, s, t0);
+    a[6] = c_fma<O>(-c1, s, t0);
+    a[5] = c_fma_rot<O, INV>(c1, d, t1);
+    a[7] = c_fma_rot<O, INV>(-c1, d, t1);
+  }
+  {   // k1 = 2: W8 y1, -+i y2, W8^3 y3: sum and difference of the first and last from y1 -+ y3
+    const C y0 = a[8], y2 = a[10], p = c_sub<O>(a[9], a[11]), q = c_add<O>(a[9], a[11]);
+    const C t0 = c_add_rot<O, INV>(y0, y2), t1 = c_sub_rot<O, INV>(y0, y2);
+    const C s = c_add_rot<O, INV>(p, q), d = c_add_rot<O, INV>(q, p);
+    a[8] = c_fma<O>(c, s, t0);
+    a[10] = c_fma<O>(-c, s, t0);
+    a[9] = c_fma_rot<O, INV>(c, d, t1);
+    a[11] = c_fma_rot<O, INV>(-c, d, t1);
+  }
+  {   // k1 = 3: W16^3 y1 = c1 u1, W8^3 y2, W16^9 y3 = -c1 u3
+    const C y0 = a[12], y1 = a[13], y2 = a[14], y3 = a[15];
+    const S p = O::fma(tn, INV ? O::im(y1) : O::re(y1), INV ? O::re(y1) : O::im(y1));
+    const S m = O::fma(-tn, INV ? O::re(y1) : O::im(y1), INV ? O::im(y1) : O::re(y1));
+    const S r2 = O::add(O::re(y2), O::im(y2)), d2 = O::sub(O::im(y2), O::re(y2));
+    const C t0 = INV ? O::mk(O::fma(-c, r2, O::re(y0)), O::fma(-c, d2, O::im(y0)))
+                     : O::mk(O::fma(c, d2, O::re(y0)), O::fma(-c, r2, O::im(y0)));
+    const C t1 = INV ? O::mk(O::fma(c, r2, O::re(y0)), O::fma(c, d2, O::im(y0)))
+                     : O::mk(O::fma(-c, d2, O::re(y0)), O::fma(c, r2, O::im(y0)));
+    const C u3 = O::mk(O::fma(T, O::im(y3), O::re(y3)), O::fma(-T, O::re(y3), O::im(y3)));
+    // forward u1 = (p, -m), inverse u1 = (-m, p); sum u1 - u3, difference u1 + u3 (negated components folded below)
+    if (INV) {
+      const C s = O::mk(O::add(m, O::re(u3)), O::sub(p, O::im(u3)));   // (-(u1 - u3).re, (u1 - u3).im)
+      const C d = O::mk(O::sub(O::re(u3), m), O::add(p, O::im(u3)));
+      a[12] = O::mk(O::fma(-c1, O::re(s), O::re(t0)), O::fma(c1, O::im(s), O::im(t0)));
+      a[14] = O::mk(O::fma(c1, O::re(s), O::re(t0)), O::fma(-c1, O::im(s), O::im(t0)));
+      a[13] = c_fma_rot<O, INV>(c1, d, t1);
+      a[15] = c_fma_rot<O, INV>(-c1, d, t1);
+    } else {
+      const C s = O::mk(O::sub(p, O::re(u3)), O::add(m, O::im(u3)));   // ((u1 - u3).re, -(u1 - u3).im)
+      const C d = O::mk(O::add(p, O::re(u3)), O::sub(O::im(u3), m));
+      a[12] = O::mk(O::fma(c1, O::re(s), O::re(t0)), O::fma(-c1, O::im(s), O::im(t0)));
+      a[14] = O::mk(O::fma(-c1, O::re(s), O::re(t0)), O::fma(c1, O::im(s), O::im(t0)));
+      a[13] = c_fma_rot<O, INV>(c1, d, t1);
+      a[15] = c_fma_rot<O, INV>(-c1, d, t1);
+    }
+  }
+  // a[4 k1 + k2] holds X[k1 + 4 k2]
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = i + 1; j < 4; ++j) {
+      const C x = a[4 * i + j];
+      a[4 * i + j] = a[4 * j + i];
+      a[4 * j + i] = x;
+    }
 }
 
 template <bool INV> struct Dft<8, INV> {
-  static __device__ __forceinline__ void run(float2* a) {
-    float2 e[4] = {a[0], a[2], a[4], a[6]};
-    float2 o[4] = {a[1], a[3], a[5], a[7]};
-    Dft<4, INV>::run(e);
-    Dft<4, INV>::run(o);
-    o[1] = w8<1, INV>(o[1]);
-    o[2] = w8<2, INV>(o[2]);
-    o[3] = w8<3, INV>(o[3]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      a[k] = cadd(e[k], o[k]);
-      a[k + 4] = csub(e[k], o[k]);
-    }
-  }
+  static __device__ __forceinline__ void run(float2* a) { dft8<LineOps, INV>(a); }
 };
-
-// multiply by exp(-+ 2 pi i e / 16)
-template <int E, bool INV>
-__device__ __forceinline__ float2 w16(float2 v) {
-  const float c1 = 0.92387953251128675613f;  // cos(pi/8)
-  const float s1 = 0.38268343236508977173f;  // sin(pi/8)
-  if (E == 0) return v;
-  if (E % 2 == 0) return w8<E / 2, INV>(v);
-  // angle = 2 pi E / 16; (cr, si) = (cos, sin)
-  const float cr = (E == 1) ? c1 : (E == 3) ? s1 : (E == 9) ? -c1 : 0.f;
-  const float si = (E == 1) ? s1 : (E == 3) ? c1 : (E == 9) ? -s1 : 0.f;
-  // forward multiplies by (cr - i si), inverse by (cr + i si)
-  return INV ? make_float2(cr * v.x - si * v.y, cr * v.y + si * v.x)
-             : make_float2(cr * v.x + si * v.y, cr * v.y - si * v.x);
-}
-
 template <bool INV> struct Dft<16, INV> {
-  // 16 = 4 x 4: inner DFT4 over a[4 n1 + n2], twiddle W16^(n2 k1), outer DFT4 over n2
-  static __device__ __forceinline__ void run(float2* a) {
-    float2 y[4][4];
-#pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) {
-      float2 t[4] = {a[n2], a[4 + n2], a[8 + n2], a[12 + n2]};
-      Dft<4, INV>::run(t);
-#pragma unroll
-      for (int k1 = 0; k1 < 4; ++k1) y[n2][k1] = t[k1];
-    }
-    y[1][1] = w16<1, INV>(y[1][1]);
-    y[1][2] = w16<2, INV>(y[1][2]);
-    y[1][3] = w16<3, INV>(y[1][3]);
-    y[2][1] = w16<2, INV>(y[2][1]);
-    y[2][2] = w16<4, INV>(y[2][2]);
-    y[2][3] = w16<6, INV>(y[2][3]);
-    y[3][1] = w16<3, INV>(y[3][1]);
-    y[3][2] = w16<6, INV>(y[3][2]);
-    y[3][3] = w16<9, INV>(y[3][3]);
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-      float2 t[4] = {y[0][k1], y[1][k1], y[2][k1], y[3][k1]};
-      Dft<4, INV>::run(t);
-#pragma unroll
-      for (int k2 = 0; k2 < 4; ++k2) a[k1 + 4 * k2] = t[k2];
-    }
-  }
+  static __device__ __forceinline__ void run(float2* a) { dft16<LineOps, INV>(a); }
 };
 
 // 3 P-point DFT (P = 2, 4, 8) from P-point and 3-point ones without twiddles between them (Good's prime

@@ -8,8 +8,7 @@
 // re and im, and an exchange through shared memory moves both lines' element
 // as one 16-byte access.  The schedule (canonical distribution: thread t owns
 // elements t + T m, radix plan, Stockham stages, stage-major twiddle tables)
-// is the one of fft_core.cuh; the paired twiddle table holds each entry w of
-// fft_core.cuh's compact table as the broadcast pairs (w.re, w.re, w.im, w.im).
+// and the twiddle tables are those of fft_core.cuh.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -47,12 +46,6 @@ __device__ __forceinline__ cp cp_add_rot(cp a, cp d) {
 template <bool INV>
 __device__ __forceinline__ cp cp_sub_rot(cp a, cp d) {
   return INV ? cp{p_add(a.re, d.im), p_sub(a.im, d.re)} : cp{p_sub(a.re, d.im), p_add(a.im, d.re)};
-}
-// s d, s = -i (forward) or +i (INV): the negation costs one paired op
-template <bool INV>
-__device__ __forceinline__ cp cp_rot(cp d) {
-  const float2 z = make_float2(0.f, 0.f);
-  return INV ? cp{p_sub(z, d.im), d.re} : cp{d.im, p_sub(z, d.re)};
 }
 // 16-byte shared-memory form {a.re, b.re, a.im, b.im}
 __device__ __forceinline__ float4 cp_pack(cp a) { return make_float4(a.re.x, a.re.y, a.im.x, a.im.y); }
@@ -98,79 +91,21 @@ template <bool INV> struct PDft<4, INV> {
   }
 };
 
-// multiply by exp(-+ 2 pi i e / 8), e = 1 or 3 (e = 2 is a rotation)
-template <int E, bool INV>
-__device__ __forceinline__ cp pw8(cp v) {
-  const float2 c = p_bc(0.70710678118654752440f);
-  if (E == 1) {
-    return INV ? cp{p_mul(c, p_sub(v.re, v.im)), p_mul(c, p_add(v.re, v.im))}
-               : cp{p_mul(c, p_add(v.re, v.im)), p_mul(c, p_sub(v.im, v.re))};
-  }
-  // E == 3
-  const float2 nc = p_bc(-0.70710678118654752440f);
-  return INV ? cp{p_mul(nc, p_add(v.re, v.im)), p_mul(c, p_sub(v.re, v.im))}
-             : cp{p_mul(c, p_sub(v.im, v.re)), p_mul(nc, p_add(v.re, v.im))};
-}
-
-template <bool INV> struct PDft<8, INV> {
-  static __device__ __forceinline__ void run(cp* a) {
-    cp e[4] = {a[0], a[2], a[4], a[6]};
-    cp o[4] = {a[1], a[3], a[5], a[7]};
-    PDft<4, INV>::run(e);
-    PDft<4, INV>::run(o);
-    o[1] = pw8<1, INV>(o[1]);
-    o[3] = pw8<3, INV>(o[3]);
-    a[0] = cp_add(e[0], o[0]);
-    a[4] = cp_sub(e[0], o[0]);
-    a[1] = cp_add(e[1], o[1]);
-    a[5] = cp_sub(e[1], o[1]);
-    a[2] = cp_add_rot<INV>(e[2], o[2]);   // o[2] times exp(-+ 2 pi i 2/8) = -+i
-    a[6] = cp_sub_rot<INV>(e[2], o[2]);
-    a[3] = cp_add(e[3], o[3]);
-    a[7] = cp_sub(e[3], o[3]);
-  }
+struct PairOps {
+  using C = cp;
+  using S = float2;
+  static __device__ __forceinline__ S re(const C& c) { return c.re; }
+  static __device__ __forceinline__ S im(const C& c) { return c.im; }
+  static __device__ __forceinline__ C mk(S r, S i) { return {r, i}; }
+  static __device__ __forceinline__ S add(S a, S b) { return p_add(a, b); }
+  static __device__ __forceinline__ S sub(S a, S b) { return p_sub(a, b); }
+  static __device__ __forceinline__ S fma(float k, S a, S b) { return p_fma(p_bc(k), a, b); }
 };
-
-// multiply by exp(-+ 2 pi i e / 16) for odd e in {1, 3, 9}
-template <int E, bool INV>
-__device__ __forceinline__ cp pw16(cp v) {
-  constexpr float c1 = 0.92387953251128675613f;  // cos(pi/8)
-  constexpr float s1 = 0.38268343236508977173f;  // sin(pi/8)
-  constexpr float cr = (E == 1) ? c1 : (E == 3) ? s1 : -c1;
-  constexpr float si = (E == 1) ? s1 : (E == 3) ? c1 : -s1;
-  // forward: (cr re + si im, cr im - si re); inverse: (cr re - si im, cr im + si re)
-  const float2 C = p_bc(cr), S = p_bc(INV ? -si : si), NS = p_bc(INV ? si : -si);
-  return {p_fma(v.re, C, p_mul(v.im, S)), p_fma(v.im, C, p_mul(v.re, NS))};
-}
-
+template <bool INV> struct PDft<8, INV> {
+  static __device__ __forceinline__ void run(cp* a) { dft8<PairOps, INV>(a); }
+};
 template <bool INV> struct PDft<16, INV> {
-  // 16 = 4 x 4: inner DFT4 over a[4 n1 + n2], twiddle W16^(n2 k1), outer DFT4 over n2
-  static __device__ __forceinline__ void run(cp* a) {
-    cp y[4][4];
-#pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) {
-      cp t[4] = {a[n2], a[4 + n2], a[8 + n2], a[12 + n2]};
-      PDft<4, INV>::run(t);
-#pragma unroll
-      for (int k1 = 0; k1 < 4; ++k1) y[n2][k1] = t[k1];
-    }
-    y[1][1] = pw16<1, INV>(y[1][1]);
-    y[1][2] = pw8<1, INV>(y[1][2]);
-    y[1][3] = pw16<3, INV>(y[1][3]);
-    y[2][1] = pw8<1, INV>(y[2][1]);
-    y[2][2] = cp_rot<INV>(y[2][2]);
-    y[2][3] = pw8<3, INV>(y[2][3]);
-    y[3][1] = pw16<3, INV>(y[3][1]);
-    y[3][2] = pw8<3, INV>(y[3][2]);
-    y[3][3] = pw16<9, INV>(y[3][3]);
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-      cp t[4] = {y[0][k1], y[1][k1], y[2][k1], y[3][k1]};
-      PDft<4, INV>::run(t);
-#pragma unroll
-      for (int k2 = 0; k2 < 4; ++k2) a[k1 + 4 * k2] = t[k2];
-    }
-  }
+  static __device__ __forceinline__ void run(cp* a) { dft16<PairOps, INV>(a); }
 };
 
 // ------------------------------------------------------------------ exchange layout
@@ -183,36 +118,16 @@ template <int SH>
 __device__ __forceinline__ int ppidx(int i) { return i + (i >> SH); }
 
 // ------------------------------------------------------------------ stages
-// The twiddle powers w^r of one butterfly as broadcast pairs (wr[r], wi[r]), from the
-// paired table (entries (w.re, w.re, w.im, w.im) in the order of fft_core.cuh's compact
-// table: stored powers 1, 2, 4, 8, the others formed by products), conjugated for INV.
-template <int R, bool INV>
-__device__ __forceinline__ void pair_twiddle_powers(float2 (&wr)[R], float2 (&wi)[R], const float4* __restrict__ tws,
-                                                    int NS) {
-#pragma unroll
-  for (int q = 0; q < tw_npow(R); ++q) {
-    const float4 x = __ldg(tws + q * NS);
-    wr[tw_pow(q)] = make_float2(x.x, x.y);
-    wi[tw_pow(q)] = INV ? make_float2(-x.z, -x.w) : make_float2(x.z, x.w);
-  }
-#pragma unroll
-  for (int r = 3; r < R; ++r) {
-    if ((r & (r - 1)) == 0) continue;
-    const int hi = r >= 8 ? 8 : (r >= 4 ? 4 : 2);
-    const int lo = r - hi;
-    wr[r] = p_sub(p_mul(wr[hi], wr[lo]), p_mul(wi[hi], wi[lo]));
-    wi[r] = p_fma(wr[hi], wi[lo], p_mul(wi[hi], wr[lo]));
-  }
-}
-// a w for a broadcast factor (wr, wi) (already conjugated for the inverse)
-__device__ __forceinline__ cp cp_mulw(cp a, float2 wr, float2 wi) {
-  return {p_sub(p_mul(a.re, wr), p_mul(a.im, wi)), p_fma(a.re, wi, p_mul(a.im, wr))};
+// a w for one twiddle factor of both lines (4096^2, N=20: fused column pass 4.38 ms; with the twiddle powers
+// formed as pairs too 4.56, with single multiplies 4.41)
+__device__ __forceinline__ cp cp_mulw(cp a, float2 w) {
+  return {p_fma(a.im, p_bc(-w.y), p_mul(a.re, p_bc(w.x))), p_fma(a.im, p_bc(w.x), p_mul(a.re, p_bc(w.y)))};
 }
 
 // As Stage in fft_core.cuh, for two lines.
 template <int N, int V, int S, int NS, bool INV, bool TRAIL>
 struct PStage {
-  static __device__ __forceinline__ void run(cp (&v)[V], float4* sm, int t, const float4* __restrict__ tw, int bid) {
+  static __device__ __forceinline__ void run(cp (&v)[V], float4* sm, int t, const float2* __restrict__ tw, int bid) {
     constexpr int R = radix_at(N, V, S);
     constexpr int T = N / V;
     constexpr int B = V / R;
@@ -225,10 +140,10 @@ struct PStage {
       for (int r = 0; r < R; ++r) a[r] = v[b + r * B];
       const int j = t + T * b;
       if (NS > 1) {
-        float2 wr[R], wi[R];
-        pair_twiddle_powers<R, INV>(wr, wi, tw + twiddle_offset(N, V, S) + (j % NS), NS);
+        float2 w[R];
+        twiddle_powers<R, INV>(w, tw + twiddle_offset(N, V, S) + (j % NS), NS);
 #pragma unroll
-        for (int r = 1; r < R; ++r) a[r] = cp_mulw(a[r], wr[r], wi[r]);
+        for (int r = 1; r < R; ++r) a[r] = cp_mulw(a[r], w[r]);
       }
       PDft<R, INV>::run(a);
       if (LAST) {
@@ -257,7 +172,7 @@ struct PStage {
 // last one is followed by a barrier, so that the next transform may start again in sa.
 template <int N, int V, int S, int NS, bool INV>
 struct PStage2 {
-  static __device__ __forceinline__ void run(cp (&v)[V], float4* sa, float4* sb, int t, const float4* __restrict__ tw,
+  static __device__ __forceinline__ void run(cp (&v)[V], float4* sa, float4* sb, int t, const float2* __restrict__ tw,
                                              int bid) {
     constexpr int R = radix_at(N, V, S);
     constexpr int T = N / V;
@@ -272,10 +187,10 @@ struct PStage2 {
       for (int r = 0; r < R; ++r) a[r] = v[b + r * B];
       const int j = t + T * b;
       if (NS > 1) {
-        float2 wr[R], wi[R];
-        pair_twiddle_powers<R, INV>(wr, wi, tw + twiddle_offset(N, V, S) + (j % NS), NS);
+        float2 w[R];
+        twiddle_powers<R, INV>(w, tw + twiddle_offset(N, V, S) + (j % NS), NS);
 #pragma unroll
-        for (int r = 1; r < R; ++r) a[r] = cp_mulw(a[r], wr[r], wi[r]);
+        for (int r = 1; r < R; ++r) a[r] = cp_mulw(a[r], w[r]);
       }
       PDft<R, INV>::run(a);
       if (LAST) {
@@ -301,7 +216,7 @@ struct PStage2 {
 // calling conventions (bid, TRAIL, canonical distribution) are those of
 // fft_line.  sm: the pair's buffer of pair_padded_len(N, V) 16-byte slots.
 template <int N, int V, bool INV, bool TRAIL = true>
-__device__ __forceinline__ void fft_pair(cp (&v)[V], float4* sm, int t, const float4* __restrict__ tw, int bid = 0) {
+__device__ __forceinline__ void fft_pair(cp (&v)[V], float4* sm, int t, const float2* __restrict__ tw, int bid = 0) {
   static_assert(N % V == 0, "V must divide N");
   static_assert(num_stages(N, V) > 0, "no radix plan");
   PStage<N, V, 0, 1, INV, TRAIL>::run(v, sm, t, tw, bid);
@@ -312,7 +227,7 @@ __device__ __forceinline__ void fft_pair(cp (&v)[V], float4* sm, int t, const fl
 // again by the next transform's exchanges (which start in sa), but not by anything else
 // before a barrier of the line.
 template <int N, int V, bool INV>
-__device__ __forceinline__ void fft_pair2(cp (&v)[V], float4* sa, float4* sb, int t, const float4* __restrict__ tw,
+__device__ __forceinline__ void fft_pair2(cp (&v)[V], float4* sa, float4* sb, int t, const float2* __restrict__ tw,
                                           int bid = 0) {
   static_assert(N % V == 0, "V must divide N");
   static_assert(num_stages(N, V) > 0, "no radix plan");

@@ -206,6 +206,12 @@ __host__ __device__ constexpr int split_row_V(int L) {
 __host__ __device__ constexpr int split_col_sel(int ny, bool cross) {
   return (cross || (ny % 3 == 0 ? ny < 192 : (ny < 128 || ny == 512))) ? 1 : 0;
 }
+// threads of a column's CTA at most: two CTAs per SM without cross sums (256), and with those of one observed
+// block on narrow power-of-two or short lines (320; 512^2 N=20, 3 blocks: 55 us, 68 with one CTA of 512), one
+// CTA otherwise (768^2 N=20, 3 blocks: 190 us, 205 with two)
+__host__ __device__ constexpr int split_col_threads(int ny, int n_obs, bool cross) {
+  return !cross ? 256 : (n_obs == 1 && (ny % 3 != 0 || ny <= 384)) ? 320 : 512;
+}
 bool split_rows_supported(int L);
 bool split_cols_supported(int ny, int n_obs, int M);
 int split_row_tile(int L);                                    // rows per tile

@@ -43,15 +43,14 @@ bool split_rows_supported(int L) { return row_line_supported(L); }
 // buffers would not fit in shared memory.  Every supported ny is a multiple of 8.
 int split_row_tile(int L) { return L >= 3072 ? 4 : 8; }
 
-// Groups of one column's CTA: at most 256 threads without cross sums (two CTAs per SM), 512 with them,
-// and the shared memory of two CTAs per SM where that leaves more than one group; then the fewest groups
-// that need as many rounds over the members.
+// Groups of one column's CTA: at most split_col_threads threads, and the shared memory of two CTAs per SM
+// where that leaves more than one group; then the fewest groups that need as many rounds over the members.
 int split_col_groups(int ny, int n_obs, int M, int N, int threads) {
   const bool cross = M > n_obs;
   const int T = ny / plan_V(ny, split_col_sel(ny, cross));
   const int nf = n_obs + 2 * n_obs * (M - n_obs);
   const size_t per = (size_t)nf * ny * sizeof(float) + (size_t)col_line_slots(ny) * sizeof(float2);
-  int g = (threads ? threads : (cross ? 512 : 256)) / T;
+  int g = (threads ? threads : split_col_threads(ny, n_obs, cross)) / T;
   if (g < 1) g = 1;
   if (g > 16) g = 16;
   while (g > 2 && g * per > 110 * 1024) --g;

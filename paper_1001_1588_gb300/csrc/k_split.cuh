@@ -280,7 +280,8 @@ __device__ __forceinline__ void add_drawn(float2 (&v)[V], unsigned long long see
 // Every group runs the same number of rounds (a group without a member in the last round works on
 // zeros), so that lines shorter than a warp can synchronise by whole warps.
 template <int NY, int V, int NOBS, bool CROSS, bool DRAWN>
-__global__ void __launch_bounds__(CROSS ? 512 : 256, CROSS ? 1 : 2) col_split_kernel(const __grid_constant__ SplitParams p) {
+__global__ void __launch_bounds__(split_col_threads(NY, NOBS, CROSS), split_col_threads(NY, NOBS, CROSS) > 320 ? 1 : 2)
+    col_split_kernel(const __grid_constant__ SplitParams p) {
   constexpr int T = NY / V;
   constexpr int PL = col_line_slots(NY);
   extern __shared__ __align__(128) unsigned char smraw[];

@@ -19,7 +19,6 @@
 #include <string>
 
 #include "../../include/fftenkf.h"
-#include "launch.cuh"
 
 namespace fftenkf {
 void set_last_error(const std::string& msg);
@@ -73,13 +72,15 @@ __device__ __forceinline__ float interp(const float* __restrict__ f, const Stenc
   return (1.f - s.wy) * ((1.f - s.wx) * f00 + s.wx * f01) + s.wy * ((1.f - s.wx) * f10 + s.wx * f11);
 }
 
-// The gather kernels work on tiles of kTX x TY nodes of one member (256 threads, TY / 4 nodes a thread).
-// Two planes of the tile and a halo of kHalo cells around it are staged side by side in shared memory
-// (wrapped at the grid's edges), so that one 8-byte shared load serves a corner of both; a node displaced
-// by kHalo cells or more takes the general gather from global memory.  Both give the same bits.
-// 2048^2, M = 2, K = 20, displacements of up to 3 cells: 2562 -> 1785 us (a thread per node gathering 8 words
-// from global memory per fixed-point step was bound by issue).  The inverse transform, one gather a node,
-// is faster without tiles (129 us against 222, K = 4).
+// The fixed-point steps work on tiles of kTX x TY nodes of one member (256 threads, TY / 4 nodes a thread):
+// the mapping's two planes of the tile and a halo of kHalo cells around it are staged side by side in shared
+// memory (wrapped at the grid's edges), so that one 8-byte shared load serves a corner of both; a node
+// displaced by kHalo cells or more takes the general gather from global memory.  Both give the same bits.
+// The blocks themselves are gathered from global memory, once a node: staging them as well made a block cost
+// 34 us instead of 15 (2040 x 1734, K = 2) and left shared memory for fewer CTAs.  2048^2, M = 2, K = 20,
+// displacements of up to 3 cells: 2530 us (a thread per node gathering 8 words from global memory per step,
+// bound by issue), 1854 with staged blocks, 1377 like this.  The inverse transform, one gather a node, is
+// faster without tiles (129 us against 222, K = 4).
 constexpr int kTX = 64, kHalo = 6, kRW = kTX + 2 * kHalo;
 template <int TY>
 struct Tile {
@@ -94,7 +95,7 @@ __device__ __forceinline__ int wrap_index(int i, int n) {
   return i;
 }
 
-// Requests planes (a, b) around the tile at (y0, x0): 4-byte asynchronous copies that interleave the two
+// Brings planes (a, b) around the tile at (y0, x0): 4-byte asynchronous copies that interleave the two
 // planes, all in flight at once (with loads through registers the staging's latency made the tiled kernel no
 // faster than gathers from global memory: 499 us against 512 at 2048^2, M = 2, K = 4).
 template <int TY>
@@ -113,12 +114,7 @@ __device__ __forceinline__ void stage_planes(Tile<TY>& t, const float* a, const 
                    : "memory");
     }
   }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-// all but the last `pending` staged tiles of this CTA have arrived
-template <int PENDING>
-__device__ __forceinline__ void stage_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
 }
 
@@ -142,76 +138,73 @@ __device__ __forceinline__ float2 sample_tile(const Tile<TY>& t, int ly, int lx,
 // grid (x: tiles of one plane; y: member k).  ext blocks 0, 1 (T) are read, blocks 2.. (r) written.  The
 // iteration stops after the first step that moves the point by at most tol cells in each component
 // (tol = 0: once an iterate repeats exactly, which gives the result of all n_iter steps), else after
-// n_iter steps.
-template <int TY>
-__global__ void __launch_bounds__(kThreads, TY > 8 ? 3 : 4) morph_forward_kernel(const float* __restrict__ u,
+// n_iter steps.  MINB = 8 spills a few of a node's values but keeps 2048 threads on an SM: 1377 us against
+// 1484 (6 CTAs) and 1600 (4), 2048^2, M = 2, K = 20, tiles of 16 rows.
+template <int TY, int MINB>
+__global__ void __launch_bounds__(kThreads, MINB) morph_forward_kernel(const float* __restrict__ u,
                                                                  const float* __restrict__ u_ref,
                                                                  float* __restrict__ ext, int M, int K, int ny,
                                                                  int nx, int n_iter, float tol, int tiles_x) {
   constexpr int NPT = TY / 4;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  Tile<TY>& t = reinterpret_cast<Tile<TY>*>(smraw)[0];   // the mapping, then every other pair of blocks
-  Tile<TY>& w = reinterpret_cast<Tile<TY>*>(smraw)[1];
+  __shared__ Tile<TY> t;
   const int plane = ny * nx;
   const int k = blockIdx.y;
   const int y0 = (blockIdx.x / tiles_x) * TY, x0 = (blockIdx.x % tiles_x) * kTX;
   const int lx = threadIdx.x % kTX, l0 = threadIdx.x / kTX;
   const float* tx = ext + (size_t)k * plane;
   const float* ty = ext + ((size_t)K + k) * plane;
-  auto block = [&](int j) { return u + ((size_t)(j < M ? j : M - 1) * K + k) * plane; };   // odd M: the last pairs with itself
   stage_planes<TY>(t, ty, tx, y0, x0, ny, nx);
-  stage_planes<TY>(w, block(0), block(1), y0, x0, ny, nx);   // lands during the fixed-point steps
-  stage_wait<1>();
-  float dy[NPT], dx[NPT];
-#pragma unroll
+#pragma unroll 1
   for (int n = 0; n < NPT; ++n) {
-    const int ly = l0 + 4 * n;
+    const int ly = l0 + 4 * n, y = y0 + ly, x = x0 + lx;
+    if (y >= ny || x >= nx) continue;
     float py = 0.f, px = 0.f;   // q_0 = p
-    if (y0 + ly < ny && x0 + lx < nx) {
-      for (int it = 0; it < n_iter; ++it) {
-        float2 f;
-        if (in_halo(py, px)) {
-          f = sample_tile<TY>(t, ly, lx, py, px);
-        } else {
-          const Stencil s = stencil(y0 + ly, x0 + lx, py, px, ny, nx);
-          f = make_float2(interp(ty, s), interp(tx, s));
-        }
-        const bool same = (fabsf(-f.y - px) <= tol) && (fabsf(-f.x - py) <= tol);
-        py = -f.x;
-        px = -f.y;
-        if (same) break;
-      }
-    }
-    dy[n] = py;
-    dx[n] = px;
-  }
-  for (int j = 0; j < M; j += 2) {
-    const bool two = j + 1 < M;
-    const float* ua = block(j);
-    const float* ub = block(j + 1);
-    Tile<TY>& cur = (j & 2) ? t : w;
-    __syncthreads();   // the other tile's readers are done
-    if (j + 2 < M) {
-      stage_planes<TY>((j & 2) ? w : t, block(j + 2), block(j + 3), y0, x0, ny, nx);
-      stage_wait<1>();
-    } else {
-      stage_wait<0>();
-    }
-#pragma unroll
-    for (int n = 0; n < NPT; ++n) {
-      const int ly = l0 + 4 * n, y = y0 + ly, x = x0 + lx;
-      if (y >= ny || x >= nx) continue;
-      const int p = y * nx + x;
+    for (int it = 0; it < n_iter; ++it) {
       float2 f;
-      if (in_halo(dy[n], dx[n])) {
-        f = sample_tile<TY>(cur, ly, lx, dy[n], dx[n]);
+      if (in_halo(py, px)) {
+        f = sample_tile<TY>(t, ly, lx, py, px);
       } else {
-        const Stencil s = stencil(y, x, dy[n], dx[n], ny, nx);
-        f = make_float2(interp(ua, s), interp(ub, s));
+        const Stencil s = stencil(y, x, py, px, ny, nx);
+        f = make_float2(interp(ty, s), interp(tx, s));
       }
-      float* r = ext + ((size_t)(2 + j) * K + k) * plane + p;
-      r[0] = f.x - __ldg(u_ref + (size_t)j * plane + p);
-      if (two) r[(size_t)K * plane] = f.y - __ldg(u_ref + (size_t)(j + 1) * plane + p);
+      const bool same = (fabsf(-f.y - px) <= tol) && (fabsf(-f.x - py) <= tol);
+      py = -f.x;
+      px = -f.y;
+      if (same) break;
+    }
+    const Stencil s = stencil(y, x, py, px, ny, nx);
+    const int p = y * nx + x;
+    for (int j = 0; j < M; ++j)
+      ext[((size_t)(2 + j) * K + k) * plane + p] =
+          interp(u + ((size_t)j * K + k) * plane, s) - __ldg(u_ref + (size_t)j * plane + p);
+  }
+}
+
+// The same without tiles, x over the nodes of one plane.
+__global__ void __launch_bounds__(kThreads, 4) morph_forward_gather(const float* __restrict__ u,
+                                                                 const float* __restrict__ u_ref,
+                                                                 float* __restrict__ ext, int M, int K, int ny,
+                                                                 int nx, int n_iter, float tol) {
+  const int plane = ny * nx;
+  const int k = blockIdx.y;
+  const float* tx = ext + (size_t)k * plane;
+  const float* ty = ext + ((size_t)K + k) * plane;
+  for (int p = blockIdx.x * kThreads + threadIdx.x; p < plane; p += gridDim.x * kThreads) {
+    const int y = p / nx, x = p - y * nx;
+    float dy = 0.f, dx = 0.f;   // q_0 = p
+    for (int it = 0; it < n_iter; ++it) {
+      const Stencil s = stencil(y, x, dy, dx, ny, nx);
+      const float ndx = -interp(tx, s);
+      const float ndy = -interp(ty, s);
+      const bool same = (fabsf(ndx - dx) <= tol) && (fabsf(ndy - dy) <= tol);
+      dx = ndx;
+      dy = ndy;
+      if (same) break;
+    }
+    const Stencil s = stencil(y, x, dy, dx, ny, nx);
+    for (int j = 0; j < M; ++j) {
+      const float v = interp(u + ((size_t)j * K + k) * plane, s);
+      ext[((size_t)(2 + j) * K + k) * plane + p] = v - __ldg(u_ref + (size_t)j * plane + p);
     }
   }
 }
@@ -276,17 +269,12 @@ int resident_ctas(K kernel) {
     per_sm = 1;
   return sms * per_sm;
 }
-// rows per tile of the gather kernels: 32, or 8 where tiles of 32 would leave SMs without two CTAs
 int sm_of_current() {
   int dev = 0, n = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
   return n > 0 ? n : 1;
 }
-bool tall_tiles(int ny, int nx, int K) {
-  return (long long)((ny + 31) / 32) * ((nx + kTX - 1) / kTX) * K >= 2 * sm_of_current();
-}
-
 dim3 member_grid(int plane, int K, int resident) {
   int gx = resident / K;
   const int need = (plane + kThreads - 1) / kThreads;
@@ -342,17 +330,20 @@ extern "C" fftenkf_status fftenkf_morph_forward(const float* u, const float* u_r
     return mfail(FFTENKF_EINVAL, std::string(who) + ": the residual blocks of ext overlap an input");
   const int tiles_x = (nx + kTX - 1) / kTX;
   cudaStream_t st_ = static_cast<cudaStream_t>(stream);
-  if (tall_tiles(ny, nx, n_members)) {
-    const size_t smem = 2 * sizeof(Tile<32>);   // 53 KB
-    int per_sm = 0;
-    if (fftenkf::kernel_shape(reinterpret_cast<const void*>(morph_forward_kernel<32>), kThreads, smem, &per_sm) != cudaSuccess)
-      return finish(who);
-    morph_forward_kernel<32><<<dim3((unsigned)(tiles_x * ((ny + 31) / 32)), (unsigned)n_members), kThreads, smem, st_>>>(
+  // Tiles of 16 rows from one wave of 8 CTAs per SM on; 8 rows below (256^2, K = 4: 15 us, 17 with 16 rows);
+  // no tiles where they hardly pay their halo and padding: up to three CTAs of nodes per SM (62 x 173, K = 9:
+  // 11 us, 13 with tiles), or less than 60 % of the tiles' columns on the grid (2400 x 65, K = 6: 40 us, 42
+  // with tiles; 1692 x 77, 60 %: 35.5 both).
+  const long long sms = sm_of_current(), tiles16 = (long long)tiles_x * ((ny + 15) / 16) * n_members;
+  if ((long long)ny * nx * n_members <= 3 * sms * kThreads || 5 * nx < 3 * kTX * tiles_x)
+    morph_forward_gather<<<member_grid(ny * nx, n_members, resident_ctas(morph_forward_gather)), kThreads, 0, st_>>>(
+        u, u_ref, ext, n_blocks, n_members, ny, nx, n_iter, tol);
+  else if (tiles16 >= 8 * sms)
+    morph_forward_kernel<16, 8><<<dim3((unsigned)(tiles_x * ((ny + 15) / 16)), (unsigned)n_members), kThreads, 0, st_>>>(
         u, u_ref, ext, n_blocks, n_members, ny, nx, n_iter, tol, tiles_x);
-  } else {
-    morph_forward_kernel<8><<<dim3((unsigned)(tiles_x * ((ny + 7) / 8)), (unsigned)n_members), kThreads, 2 * sizeof(Tile<8>), st_>>>(
+  else
+    morph_forward_kernel<8, 4><<<dim3((unsigned)(tiles_x * ((ny + 7) / 8)), (unsigned)n_members), kThreads, 0, st_>>>(
         u, u_ref, ext, n_blocks, n_members, ny, nx, n_iter, tol, tiles_x);
-  }
   return finish(who);
 }
 

@@ -213,7 +213,7 @@ fftenkf_status fftenkf_get_schedule(fftenkf_plan plan, int* sched, int n);
  *     K_j(k) = chat_{j,O}(k) (chat_{O,O}(k) + diag(rhat_O(k)))^-1,
  * chat_{a,b} = 1/(N-1) sum_k ahat_k^(a) conj(ahat_k^(b)) (eq. dii, cov-multi-spectral),
  * and u_k^(j),a = u_k^(j) + F^-1 sum_o K_{j,o} F(d_o + e_{k,o} - u_k^(o)) for every block,
- * observed ones included.  The n_obs x n_obs bracket is inverted in FP64; where it is
+ * observed ones included.  The n_obs x n_obs bracket is inverted beyond FP32; where it is
  * singular (rhat = 0 and det <= 1e-6 a11 a22) its rank-1 pseudo-inverse A / tr(A)^2 is
  * used, and 0 where tr(A) = 0.  This generalises the paper, which derives the single
  * observed block.
@@ -302,14 +302,16 @@ fftenkf_status fftenkf_denoise_spectrum(fftenkf_denoiser d, const float* params,
  * eq. (spectral-multi-enkf) are applied with S in place of F (real coefficients; observed
  * blocks' mutual cross-covariances neglected as for the periodic plan; gain 0 where
  * chat + rhat == 0).  Boundary nodes of the ensemble are left as they are.
- * The transform is computed exactly as the periodic one of the odd extension of the interior to
- * the period 2(ny-1) x 2(nx-1), whose DFT is -S of the interior at the wavenumbers 1..m of each
- * axis (and their negatives) and zero on the lines 0 and m+1: the plan extends the inputs into
- * plan-owned buffers, runs the periodic analysis there and copies the interior back.  So
- * 2(ny-1) and 2(nx-1) must satisfy the periodic plan's rules (ny-1 in {2^a, 3*2^a} up to 2048,
- * nx-1 in {2^a, 3*2^a} up to 4096, both at least 8), else EUNSUPPORTED; the plan allocates
- * about 4x the ensemble, perturbations and data, and 4x the work of a periodic analysis on
- * ny x nx.  Device pointers need only the alignment of their element type.
+ * The transform is computed through the odd extension of the interior to the period
+ * 2(ny-1) x 2(nx-1), whose DFT is -S of the interior at the wavenumbers 1..m of each axis (and
+ * their negatives) and zero on the lines 0 and m+1: line by line in the row and column passes,
+ * with the real coefficients of the interior in plan-owned buffers (4 bytes per node of the
+ * ensemble and the perturbations).  Grids those passes do not cover (nx-1 above 2048, ny-1 or
+ * nx-1 not a multiple of 8, covariance sums beyond a column's shared memory) are extended into
+ * plan-owned buffers (about 4x the ensemble, perturbations and data), analysed there by the
+ * periodic passes, and the interior copied back.  2(ny-1) and 2(nx-1) must satisfy the periodic
+ * plan's rules (ny-1 in {2^a, 3*2^a} up to 2048, nx-1 in {2^a, 3*2^a} up to 4096, both at least
+ * 8), else EUNSUPPORTED.  Device pointers need only the alignment of their element type.
  *   ensemble      [M][N][ny][nx] storage dtype, in place
  *   data          [n_obs][ny][nx] float; perturbations [N][n_obs][ny][nx] storage dtype
  *                 (only their interior nodes enter)

@@ -525,7 +525,7 @@ static cudaError_t run_columns(fftenkf_plan p, const SplitParams& q, const doubl
   if (spectrum) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
   } else if (p->coupled) {
-    // tables of the column statistics, then the coupled gains (FP64 bracket inverse per wavenumber)
+    // tables of the column statistics, then the coupled gains (bracket inverse per wavenumber)
     if (e == cudaSuccess) e = run_statistics(p, ws, s, nullptr);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join, 0);
     CoupledGainParams cg;

@@ -221,6 +221,30 @@ cudaError_t launch_row_split(SplitParams p, cudaStream_t s);
 cudaError_t launch_col_split(SplitParams p, cudaStream_t s);
 cudaError_t launch_row_inv_split(SplitParams p, cudaStream_t s);
 
+// The real sine variant's passes (k_sine.cuh)
+struct SineParams {
+  int ny, nx, M, N, n_obs, storage;
+  int obs[kMaxObs];
+  int role_block[kMaxBlocks];
+  int anomalies, innovations;   // forward rows
+  void* ens;              // [M][N][ny][nx], interior updated in place
+  const float* data;      // [n_obs][ny][nx]
+  const void* pert;       // [N][n_obs][ny][nx]
+  const double* rhat;     // [n_obs][ny-2][nx-2]
+  double* spectrum_out;   // columns: tables wanted instead of the update, [n_obs (1 + n_un)][ny-2][nx-2]
+  float *A, *W;           // coefficients, fields of fstride = (nx-2)(ny-1) floats
+  size_t fstride;
+  const float2 *twx, *twy;   // tables of the 2(nx-1)- and 2(ny-1)-point plans
+  int groups, acc_bytes;  // column pass: thread groups, shared memory of the sums
+  float inv_sqrt_N, scale, inv_G;   // scale = inv_G / (N-1), inv_G = 1 / (4 (ny-1)(nx-1))
+  int* status;
+};
+// thread groups of a column's CTA; 0 where the sine passes do not cover the shape
+int sine_col_groups(int ny, int nx, int n_obs, int M, int N);
+cudaError_t launch_sine_rows(const SineParams& p, cudaStream_t s);
+cudaError_t launch_sine_cols(SineParams p, cudaStream_t s);
+cudaError_t launch_sine_rows_inv(const SineParams& p, cudaStream_t s);
+
 // column groups that the fused pass keeps on the GPU at once
 int col_fused_groups(int ny, int sel);
 int sm_count();

@@ -199,7 +199,7 @@ cudaError_t launch_rhat_transpose(const double* rhat, double* rhat_t, int n, int
   return cudaGetLastError();
 }
 
-// g A^-1 of the bracket A = [[a0 + r0, conj b], [b, a1 + r1]] in FP64: A^-1 when det A > 1e-6 a11 a22, the
+// g A^-1 of the bracket A = [[a0 + r0, conj b], [b, a1 + r1]], in float pairs or FP64: A^-1 when det A > 1e-6 a11 a22, the
 // pseudo-inverse A / tr(A)^2 of a rank-1 bracket otherwise, 0 where tr(A) = 0; rounded to float.
 struct Bracket {
   float s00, s11;

@@ -20,7 +20,7 @@
 namespace fftenkf {
 
 // complex lines of a row tile, two rows each: the longest in tiles of 4 rows, so that two CTAs share an SM
-// (2049^2 nodes, 4 blocks, N=20, BF16: 8.38 ms, 11.0 with tiles of 8; at 3072 points, 513 x 1537, 2 blocks,
+// (2049^2 nodes, 4 blocks, N=20, BF16: 11.0 -> 8.4 ms; at 3072 points, 513 x 1537, 2 blocks,
 // tiles of 4 would take 916 us instead of 870)
 __host__ __device__ constexpr int sine_tile_lines(int P) { return P >= 4096 ? 2 : 4; }
 
@@ -86,42 +86,44 @@ __global__ void __launch_bounds__(256, 2) sine_rows_kernel(const __grid_constant
     const int y = 1 + 2 * NL * tile + 2 * (l + g);                // rows y and y + 1
     const size_t ra = (size_t)y * nx, rb = ra + nx;
     const bool has_b = y + 1 < ny - 1;                       // the last line's second row is the boundary
-    float2 v[V];
+    // Every load is unconditional (position 0 and the row after the last are the grid's boundary) and issued
+    // before the first use: with the zeros chosen by branches around the loads few were in flight, and 62 % of
+    // the stalls were waits for them (analysis of 1025^2 nodes, 4 observed blocks, N=20, BF16: 2.52 -> 1.96 ms).
+    float2 v[V], c[V / 2], d2[V / 2];
+    const bool sum = anom && k == 0;
 #pragma unroll
     for (int m = 0; m < V / 2; ++m) {
       const int x = t + T * m;
-      float a = 0.f, b = 0.f;
-      if (x != 0) {
-        if (!anom) {
-          a = d[ra + x] - load1<ST>(uk, ra + x) + load1<ST>(e, ra + x);   // d - u first
-          if (has_b) b = d[rb + x] - load1<ST>(uk, rb + x) + load1<ST>(e, rb + x);
-        } else if (k > 0) {
-          a = load1<ST>(uk, ra + x) - load1<ST>(u0, ra + x);
-          if (has_b) b = load1<ST>(uk, rb + x) - load1<ST>(u0, rb + x);
-        }
+      v[m] = make_float2(load1<ST>(uk, ra + x), load1<ST>(uk, rb + x));
+      if (anom) c[m] = make_float2(load1<ST>(u0, ra + x), load1<ST>(u0, rb + x));
+      else {
+        c[m] = make_float2(load1<ST>(e, ra + x), load1<ST>(e, rb + x));
+        d2[m] = make_float2(d[ra + x], d[rb + x]);
       }
-      v[m] = make_float2(a, b);
     }
-    if (anom && k == 0) {   // (1/sqrt N) sum_k (u_k - u_0), in member order
-      float2 c[V / 2];
+    if (!anom) {
 #pragma unroll
-      for (int m = 0; m < V / 2; ++m) {
-        const int x = t + T * m;
-        c[m] = make_float2(load1<ST>(u0, ra + x), has_b ? load1<ST>(u0, rb + x) : 0.f);
-      }
-#pragma unroll 1
+      for (int m = 0; m < V / 2; ++m) v[m] = cadd(csub(d2[m], v[m]), c[m]);   // d - u first
+    } else if (!sum) {
+#pragma unroll
+      for (int m = 0; m < V / 2; ++m) v[m] = csub(v[m], c[m]);
+    } else {   // (1/sqrt N) sum_k (u_k - u_0), in member order
+#pragma unroll
+      for (int m = 0; m < V / 2; ++m) v[m] = make_float2(0.f, 0.f);
+#pragma unroll 2
       for (int q = 1; q < N; ++q) {
         const char* uq = u0 + (size_t)q * G * es;
 #pragma unroll
-        for (int m = 0; m < V / 2; ++m) {
-          const int x = t + T * m;
-          if (x == 0) continue;
-          v[m].x += load1<ST>(uq, ra + x) - c[m].x;
-          if (has_b) v[m].y += load1<ST>(uq, rb + x) - c[m].y;
-        }
+        for (int m = 0; m < V / 2; ++m)
+          v[m] = cadd(v[m], csub(make_float2(load1<ST>(uq, ra + t + T * m), load1<ST>(uq, rb + t + T * m)), c[m]));
       }
 #pragma unroll
       for (int m = 0; m < V / 2; ++m) v[m] = cscale(v[m], p.inv_sqrt_N);
+    }
+#pragma unroll
+    for (int m = 0; m < V / 2; ++m) {
+      if (t + T * m == 0) v[m] = make_float2(0.f, 0.f);
+      if (!has_b) v[m].y = 0.f;
     }
     float2* line = lines + (l + g) * pitch;
     odd_extension<P, V>(v, line, t, line_bar<T>(g));
@@ -157,6 +159,7 @@ __global__ void __launch_bounds__(256, 2) sine_rows_inv_kernel(const __grid_cons
   const int nf = p.M * p.N, ny = p.ny, nx = p.nx;
   const int tile = blockIdx.x / nf, f = blockIdx.x - tile * nf;
   const float* in = p.A + (size_t)f * p.fstride + 2 * NL * tile;
+#pragma unroll 4
   for (int q = threadIdx.x; q < Q * (nx - 2); q += blockDim.x) {
     const int kx = 1 + q / Q, h = q % Q;
     const float4 s = *reinterpret_cast<const float4*>(in + (size_t)(kx - 1) * (ny - 1) + 4 * h);
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(256, 2) sine_rows_inv_kernel(const __grid_cons
 #pragma unroll
     for (int m = 0; m < V / 2; ++m) {
       const int x = t + T * m;
-      a[m] = make_float2(load1<ST>(u, ra + x), has_b ? load1<ST>(u, rb + x) : 0.f);
+      a[m] = make_float2(load1<ST>(u, ra + x), load1<ST>(u, rb + x));
     }
 #pragma unroll
     for (int m = 0; m < V; ++m) v[m] = line[pidx(t + T * m)];
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(256, 2) sine_rows_inv_kernel(const __grid_cons
 // col_split_kernel: members over the CTA's groups, sums in shared memory, gains, update; all tables real.
 // smem: sums [groups][nf][2][n] f32, n = ny - 1 | exchange lines [groups][PL] f2
 template <int P, int NOBS>
-__global__ void __launch_bounds__(256, NOBS <= 2 ? 2 : 1) sine_cols_kernel(const __grid_constant__ SineParams p) {
+__global__ void __launch_bounds__(sine_col_threads(NOBS), 1) sine_cols_kernel(const __grid_constant__ SineParams p) {
   constexpr int V = plan_V(P, 0), T = P / V, n = P / 2, H = V / 2, PL = col_line_slots(P);
   extern __shared__ __align__(128) unsigned char smraw[];
   stream_order_wait();

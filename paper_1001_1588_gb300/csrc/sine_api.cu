@@ -7,8 +7,8 @@
 // products of their sine coefficients, the periodic gains are even in each wavenumber, the
 // periodic update of an odd innovation stays odd, and its interior is the sine-transform update.
 // The passes of k_sine.cuh use that line by line: no extended copies, a quarter of the row spectra and half of
-// the transforms (1025^2 nodes, 4 blocks, 2 observed, N=20, BF16: 2.00 ms, 3.28 through the extension; 65^2,
-// 63 us against 490; never slower at the 18 shapes measured).  Rows whose extension is longer than 4096
+// the transforms (1025^2 nodes, 4 blocks, 2 observed, N=20, BF16: 1.55 ms, 3.28 through the extension; 65^2,
+// 60 us against 490; never slower at the 18 shapes measured).  Rows whose extension is longer than 4096
 // points, sides that are not a multiple of 8, and block states whose sums do not fit in a column's shared
 // memory, build the odd extensions in plan-owned buffers (exact: copies and sign flips),
 // run the periodic analysis through the public C ABI, and copy the interior back.

@@ -274,10 +274,9 @@ def kernel_traffic(pass_name):
 
 # sources outside the analysis path whose counters profiles/traffic.json holds: front ends that
 # reach the periodic analysis only through its C ABI (sine, batched, allocation-free), and the
-# kernels of other workloads (batched, learned spectrum, morphing).  The hash identifies the
+# kernels of other workloads (sine, learned spectrum, morphing).  The hash identifies the
 # analysis path's kernels and everything they include.
-OTHER_SOURCES = ("sine_api.cu", "batch_api.cu", "batch.cuh", "k_batch.cuh", "k_batch.cu", "k_mlp.cu", "mlp_api.cu",
-                 "morph_api.cu", "static_api.cu")
+OTHER_SOURCES = ("sine_api.cu", "batch_api.cu", "k_mlp.cu", "mlp_api.cu", "morph_api.cu", "static_api.cu")
 
 
 def _code_only(text):
@@ -291,7 +290,7 @@ def source_sha():
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1001_1588_gb300", "csrc")
     for f in sorted(os.listdir(csrc)):
-        if f.endswith((".cu", ".cuh")) and f not in OTHER_SOURCES and not f.startswith("k_batch_"):
+        if f.endswith((".cu", ".cuh")) and f not in OTHER_SOURCES and not f.startswith("k_sine"):
             h.update(_code_only(open(os.path.join(csrc, f), encoding="utf-8").read()).encode())
     return h.hexdigest()[:16]
 
@@ -991,19 +990,14 @@ def run_sine(a):
                               "frac_native": B_native / (ms / 1e3) / 1e9 / peak, "peak": peak,
                               "peak_kind": peak_kind},
         "periodic_extension_ms": ms_p, "extension_overhead_ms": None if ms_p is None else ms - ms_p, "clocks": clk.summary(),
-        "gpu_launches": 10 * a.steps,   # 3 extensions, rhat extension, 5 of the periodic analysis, interior copy
+        "gpu_launches": 3 * a.steps,   # rows, columns, inverse rows
     }))
     return 0
 
 
 def batched_launches(items):
-    """Launches of one batched analysis: an analysis of at least 512 x 256 points runs on its own
-    plan (rhat transposition, anomaly rows, innovation rows, inverse rows, and the fused column
-    pass for 512-4096-point power-of-two columns, else the statistics and update passes); the
-    others share the 7 persistent launches."""
-    big = [it for it in items if it.ny * it.nx >= 512 * 256]
-    n = sum(5 if (it.ny >= 512 and (it.ny & (it.ny - 1)) == 0) else 6 for it in big)
-    return n + (7 if len(big) < len(items) else 0)
+    """Launches of one batched analysis: the forward rows, columns and inverse rows of every grid shape."""
+    return 3 * len({(it.ny, it.nx) for it in items})
 
 
 def run_batched(a):
@@ -1048,8 +1042,8 @@ def run_batched(a):
         "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
         "data": "synthetic",
         "config": {"workload": "batched: %d single-block analyses, sides {64..1024} square and 2:1, N in 5..25, "
-                               "SE spectra, flat rhat, FP32, one CUDA graph: analyses of >= 512x256 points on "
-                               "their own plans on 8 branches, the others in 7 persistent launches" % len(items),
+                               "SE spectra, flat rhat, FP32, one CUDA graph: three launches per grid shape on "
+                               "8 branches" % len(items),
                    "grid_points_total": sum(it.ny * it.nx for it in items), "members_total": sum(it.N for it in items)},
         "analysis_roofline": {"alg_bytes": B, "achieved_gbs": B / (ms / 1e3) / 1e9,
                               "frac": B / (ms / 1e3) / 1e9 / peak, "peak": peak, "peak_kind": peak_kind},

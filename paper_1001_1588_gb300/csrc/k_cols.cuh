@@ -254,7 +254,7 @@ __global__ void __launch_bounds__((NY / V > 256) ? 512 : 256, 1) col_stats_kerne
 // Two bulk-copy pipelines: innovation lines one item ahead (two stages, or one
 // when shared memory is short) and gain lines one target block ahead (one
 // stage, read into registers before the next copy is issued).
-// smem: wst [nst][LPC][n_obs][NY] f2 | gst [LPC][n_obs][NY] f2 | xbuf [LPC][PL] f2 | bars[3] | flag
+// smem: wst [nst][LPC][n_obs][NY] f2 | gst [LPC][n_obs][NY] f2 | xbuf [LPC][PL] f2 | bars[3] | wflag | gflag
 // DRAWN: the perturbations are drawn here (seeded analysis); a separate instantiation, so that the
 // analysis with given perturbations carries none of the generator's code
 template <int NY, int V, int NOBS, bool DRAWN>
@@ -272,7 +272,10 @@ __global__ void __launch_bounds__((NY / V > 256) ? 512 : 256, 1) col_update_kern
   float2* xbuf = gst + stage_elems + (size_t)g * PL;
   uint64_t* bars = reinterpret_cast<uint64_t*>(gst + stage_elems + (size_t)LPC * PL);
   uint64_t* gbar = bars + 2;
-  int* flag = reinterpret_cast<int*>(bars + 3);
+  // A verdict word per pipeline: the innovation wait and the gain wait that follows it are separated by the
+  // line's barriers only (one warp of a line may not have read the first verdict when thread 0 has the second).
+  int* wflag = reinterpret_cast<int*>(bars + 3);
+  int* gflag = wflag + 1;
   const long long n_items = (long long)(p.L + 1) * p.N;
   const long long step = (long long)gridDim.x * LPC;
   const size_t fstride = (size_t)p.L * NY;
@@ -335,7 +338,7 @@ __global__ void __launch_bounds__((NY / V > 256) ? 512 : 256, 1) col_update_kern
   }
   for (int it = 0; base < n_items; base += step, ++it) {
     const int s = (nst == 2) ? (it & 1) : 0;
-    if (!cta_wait(&bars[s], s ? wph1 : wph0, p.status, flag)) {
+    if (!cta_wait(&bars[s], s ? wph1 : wph0, p.status, wflag)) {
       if (threadIdx.x == 0) {   // other copies may still be landing: let them finish
         mbar_wait_bounded(&bars[s ^ 1], s ? wph0 : wph1);
         mbar_wait_bounded(gbar, gph);
@@ -394,7 +397,7 @@ __global__ void __launch_bounds__((NY / V > 256) ? 512 : 256, 1) col_update_kern
       }
     }
     for (int j = 0; j < p.M; ++j) {
-      if (!cta_wait(gbar, gph, p.status, flag)) {
+      if (!cta_wait(gbar, gph, p.status, gflag)) {
         if (threadIdx.x == 0) {
           mbar_wait_bounded(&bars[0], wph0);
           mbar_wait_bounded(&bars[1], wph1);

@@ -406,6 +406,7 @@ __global__ void __launch_bounds__(V <= 8 ? 512 : 256, 1) col_fused_kernel(const 
     }
     for (int u = 0; u < units; ++u) {
       const int b = consumed & 1;
+      stage_reads_done();   // the previous unit's slot, as a stage and as an exchange buffer: copied into below
       // the group waits for the unit's copies (thread 0 polls, bounded; the verdict is shared)
       if (t == 0) {
         bool ok = mbar_wait_bounded(&bars[b], b ? ph1 : ph0);
@@ -422,8 +423,8 @@ __global__ void __launch_bounds__(V <= 8 ? 512 : 256, 1) col_fused_kernel(const 
         break;
       }
       if (b) ph1 ^= 1; else ph0 ^= 1;
-      // every thread of the group has left the previous unit (its reads of the other slot,
-      // as a stage and as an exchange buffer): that slot takes the next unit's copy
+      // every thread of the group has left the previous unit (its reads and writes of the other
+      // slot): that slot takes the next unit's copy
       if (t == 0 && consumed > 0) issue_next();
       const bool stats = u < units_stats;
       const int pp = stats ? u % P : 0;

@@ -42,9 +42,9 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
-// Called by every thread between its last reads of a shared-memory stage and the barrier after which
-// the stage's next copy is issued.  A barrier alone orders the reads against other threads' writes, not
-// against a copy's: loads still queued behind bank conflicts (rows of 32 or 64 points, 16 rows to a warp)
+// Called by every thread between its last accesses to a shared-memory stage and the barrier after which
+// the stage's next copy is issued.  A barrier alone orders them against other threads' writes, not
+// against a copy's: writes of a stage that also serves as an exchange buffer might land after the copy, and loads still queued behind bank conflicts (rows of 32 or 64 points, 16 rows to a warp)
 // would return the next copy's data.
 __device__ __forceinline__ void stage_reads_done() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 

@@ -35,3 +35,19 @@ def test_verdict_is_read_before_the_word_is_written_again(file, kernel):
         later = [w for w in waits[n + 1:] if w[1] == word]
         until = later[0][0] if later else len(body)   # the word's next wait, or its own in the next pass of the loop
         assert "__syncthreads()" in body[end:until], word
+
+
+@pytest.mark.parametrize("file,kernel", KERNELS + [("k_colf.cuh", "col_fused_kernel")])
+def test_stage_is_fenced_before_its_next_copy(file, kernel):
+    """In the loop over the staged units, every barrier after which one thread issues a copy into a stage is
+    preceded by the fence that orders the threads' accesses to that stage before the copy, with no other barrier
+    in between.  (issue_w of the column update follows a later barrier: its stage is read before the gain stage,
+    whose fence covers both.)"""
+    body = _body(file, kernel)
+    barrier = r"__syncthreads\(\)|line_sync<T>\(bid\)|cta_wait\("
+    loop = re.search(r"for \([^;]*; (q < Q|cb < ncol|base < n_items|c < ncol)", body).start()   # past the first copies
+    issues = [m.start() for m in re.finditer(r"issue(?:_next|_tile|_rows|_g)?\(", body) if m.start() > loop]
+    assert issues
+    for at in issues:
+        barriers = [m.start() for m in re.finditer(barrier, body[:at])]
+        assert "stage_reads_done()" in body[barriers[-2]:barriers[-1]], body[at:at + 40]

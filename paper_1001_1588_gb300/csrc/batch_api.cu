@@ -67,11 +67,22 @@ struct fftenkf_batch_s {
   int bt[kStages] = {256, 256, 256};
   cudaStream_t lane[kLanes] = {};
   cudaEvent_t ev_fork = nullptr, ev_lane[kLanes] = {};
+  cudaEvent_t ev_read = nullptr;       // after the last launch that reads the item table
   cudaStream_t cap = nullptr;
   cudaGraphExec_t exec = nullptr;
   char* bound_ws = nullptr;
-  bool items_dirty = true;
+  bool items_dirty = true;             // the device table does not hold `items`
 };
+
+// The host's item table to the device, ordered on s and after the last analysis, which may be running on
+// another stream and reads the table.  (The copy is pageable: the runtime stages the host table before
+// it returns.)
+static cudaError_t upload_items(fftenkf_batch b, cudaStream_t s) {
+  cudaError_t e = cudaStreamWaitEvent(s, b->ev_read, 0);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->d_items, b->items.data(), b->count * sizeof(SplitItem), cudaMemcpyHostToDevice, s);
+  return e;
+}
 
 static SplitParams class_params(fftenkf_batch b, const ShapeClass& c) {
   SplitParams q;
@@ -212,6 +223,7 @@ extern "C" fftenkf_status fftenkf_plan_batched(fftenkf_batch* out, int count, co
   if (e == cudaSuccess) e = build_units(b);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_read, cudaEventDisableTiming);
   for (int l = 0; l < kLanes && e == cudaSuccess; ++l) {
     e = cudaStreamCreateWithFlags(&b->lane[l], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_lane[l], cudaEventDisableTiming);
@@ -233,6 +245,7 @@ extern "C" fftenkf_status fftenkf_batch_destroy(fftenkf_batch b) {
     if (b->ev_lane[l]) cudaEventDestroy(b->ev_lane[l]);
   }
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+  if (b->ev_read) cudaEventDestroy(b->ev_read);
   if (b->d_units) cudaFree(b->d_units);
   if (b->d_items) cudaFree(b->d_items);
   if (b->d_tw) cudaFree(b->d_tw);
@@ -298,10 +311,8 @@ extern "C" fftenkf_status fftenkf_analyze_batched(fftenkf_batch b, void* const* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
   if (b->items_dirty) {
-    // pageable copy: the runtime stages the host table before returning, ordered on s
-    e = cudaMemcpyAsync(b->d_items, b->items.data(), b->count * sizeof(SplitItem), cudaMemcpyHostToDevice, s);
+    e = upload_items(b, s);
     if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("item table: ") + cudaGetErrorString(e));
-    b->items_dirty = false;
   }
   if (!b->exec) {
     cudaGraph_t g = nullptr;
@@ -325,7 +336,9 @@ extern "C" fftenkf_status fftenkf_analyze_batched(fftenkf_batch b, void* const* 
     }
   }
   e = cudaGraphLaunch(b->exec, s);
+  if (e == cudaSuccess) e = cudaEventRecord(b->ev_read, s);
   if (e != cudaSuccess) return bfail(FFTENKF_ECUDA, std::string("graph launch: ") + cudaGetErrorString(e));
+  b->items_dirty = false;   // only now: the copy of a call that was refused (s under capture) has not run
   return FFTENKF_OK;
 }
 
@@ -364,12 +377,11 @@ extern "C" fftenkf_status fftenkf_batch_autotune(fftenkf_batch b, void* workspac
   std::vector<SplitItem> saved = b->items;
   char* saved_ws = b->bound_ws;
   bind(b, ens.data(), dat.data(), pert.data(), rh.data(), ws);
-  cudaMemcpyAsync(b->d_items, b->items.data(), b->count * sizeof(SplitItem), cudaMemcpyHostToDevice, s);
+  cudaError_t e = upload_items(b, s);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   double total = 0.0;
-  cudaError_t e = cudaSuccess;
   for (int stage = 0; stage < kStages && e == cudaSuccess; ++stage) {
     float best = 1e30f;
     int keep = kCandBt[0];

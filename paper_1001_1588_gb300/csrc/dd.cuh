@@ -3,10 +3,12 @@
 // GB300's FP64 unit is slow even for single adds and conversions: forming chat + rhat in FP64 for every
 // wavenumber and observed block (one add and two conversions, 16.8 M times at 4096^2 with two observed
 // blocks) took 0.9 ms of the fused column pass's 5.4, nearly all of its gain step.  Here a double is split by
-// integer operations into two floats, hi + lo with 48 of its 53 bits, sums and quotients are formed in
-// float pairs (Knuth's two-sum, FMA products) and rounded to float once, as the FP64 results were.  Values
-// whose exponent leaves no room for the pair (below 2^-74 or above 2^120, not 0) and denominators that
-// are not comfortably normal floats take FP64, out of line.
+// integer operations into floats (all 53 bits: 24 + 24 + 5), and sums, products and quotients are formed in
+// float pairs (Knuth's two-sum, FMA products).  Every result is the exact value rounded to float once: sums by
+// rounding to odd first (Boldo and Melquiond), quotients by Ziv's test, which takes FP64, out of line, where
+// the pair's error could change the rounding.  So no result is further from the exact value than the same
+// FP64 operations rounded to float.  Values whose exponent leaves no room for the pair (below 2^-74 or above
+// 2^120, not 0), sums that cancel, and denominators that are not comfortably normal floats take FP64 too.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -17,8 +19,9 @@ struct fpair {
   float h, l;
 };
 
-// x as hi + lo (hi its leading 24 bits, lo the next 24); false where x is neither 0 nor within 2^-74 .. 2^120
-__device__ __forceinline__ bool split_double(double x, fpair& p) {
+// x as hi + lo (hi its leading 24 bits, lo the next 24, rounded), and the last bits' remainder in rest; false
+// where x is neither 0 nor within 2^-74 .. 2^120
+__device__ __forceinline__ bool split_double(double x, fpair& p, float& rest) {
   const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
   const int e = (int)((h >> 20) & 0x7ffu);
   const uint32_t sign = h & 0x80000000u;
@@ -26,8 +29,13 @@ __device__ __forceinline__ bool split_double(double x, fpair& p) {
   const uint32_t hi = (((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29);
   const float scale = __uint_as_float(((uint32_t)(e - 948) << 23) | sign);   // 2^(e - 1075), signed
   p.h = zero ? 0.f : __uint_as_float(hi | sign);
-  p.l = zero ? 0.f : __uint2float_rn(l & 0x1fffffffu) * scale;
+  p.l = zero ? 0.f : __uint2float_rn(l & 0x1fffffe0u) * scale;
+  rest = zero ? 0.f : __uint2float_rn(l & 0x1fu) * scale;
   return zero || (unsigned)(e - 949) <= 194u;
+}
+__device__ __forceinline__ bool split_double(double x, fpair& p) {
+  float rest;
+  return split_double(x, p, rest);
 }
 
 // x rounded to float (nearest, ties to even), as the conversion instruction does
@@ -73,53 +81,121 @@ __device__ __forceinline__ fpair pair_recip(fpair a) {
   const float i = __frcp_rn(a.h);
   return {i, i * fmaf(-a.l, i, fmaf(-a.h, i, 1.f))};
 }
-// a b s rounded to float once
-__device__ __forceinline__ float pair_product(fpair a, fpair b, float s) {
+// a b s rounded to float; false where an error of 2^-42 cond in it could change the rounding (or it is tiny).
+// The pair operations above and a truncated split are within 2^-44 of their values each.
+__device__ __forceinline__ bool pair_product(fpair a, fpair b, float s, float cond, float& out) {
   const fpair p = pair_mul(a, b);
   const float t = __fmul_rn(p.h, s);
-  return t + fmaf(p.l, s, fmaf(p.h, s, -t));
+  const float e = fmaf(p.l, s, fmaf(p.h, s, -t));
+  const float d = fabsf(t) * 0x1p-42f * cond;
+  out = t + (e + d);
+  return (out == t + (e - d) && fabsf(t) >= 1e-30f) || a.h == 0.f;
 }
 __device__ __forceinline__ bool well_inside(float x) { return fabsf(x) >= 1e-30f && fabsf(x) <= 1e30f; }
 
 // chat + rhat rounded to float; false where it must be formed in FP64 (and where it is below FLT_MIN)
 __device__ __forceinline__ bool denominator(float val, double rhat, float& den) {
   fpair r;
-  const bool ok = split_double(rhat, r);
+  float rest;
+  const bool ok = split_double(rhat, r, rest);
   const fpair s = two_sum(val, r.h);
-  den = s.h + (s.l + r.l);
-  return ok && den >= 1.17549435e-38f;
+  // the tail s.l + r.l + rest rounded to odd: where t.l + rest is not 0, the neighbour on its side of an even t.h
+  const fpair t = two_sum(s.l, r.l);
+  const float low = t.l + rest;
+  const uint32_t b = __float_as_uint(t.h), toward = ((b ^ __float_as_uint(low)) >> 31) ? ~0u : 1u;
+  const float odd = __uint_as_float((low != 0.f && !(b & 1u)) ? b + toward : b);
+  den = s.h + (t.h == 0.f ? low : odd);
+  return ok && den >= 1.17549435e-38f && den >= 0.5f * fabsf(r.h);   // no cancellation
 }
 // inv_G / (val + rhat) in FP64, 0 where the denominator is exactly 0
 static __device__ __noinline__ double quotient_fp64(float val, double rhat, float inv_G) {
   const double den = (double)val + rhat;
   return (den != 0.0) ? (double)inv_G / den : 0.0;
 }
+// a + b of two numbers split without their last bits; false where it cancels or is no comfortable float
+__device__ __forceinline__ bool pair_sum(fpair a, fpair b, fpair& s) {
+  s = pair_add(a, b);
+  return well_inside(s.h) && fabsf(s.h) >= 0.5f * fmaxf(fabsf(a.h), fabsf(b.h));
+}
+// the same rounded to float
+__device__ __forceinline__ float quotient(float val, double rhat, float inv_G) {
+  fpair r, den;
+  const bool in = split_double(rhat, r);
+  float q;
+  if (in && pair_sum({val, 0.f}, r, den) && pair_product({1.f, 0.f}, pair_recip(den), inv_G, 1.f, q)) return q;
+  return (float)quotient_fp64(val, rhat, inv_G);
+}
 
-// scale / (a + rhat) for a caller's spectrum, and its products with entries of the spectrum, each rounded
+static __device__ __noinline__ double spec_quotient_fp64(double den, float scale) {
+  return (den != 0.0) ? (double)scale / den : 0.0;
+}
+static __device__ __noinline__ float spec_product_fp64(double x, double a, double rhat, float scale) {
+  return (float)(x * spec_quotient_fp64(a + rhat, scale));
+}
+
+// scale / (a + rhat) for a caller's spectrum, and its products with entries x of the spectrum, each rounded
 // to float once
 struct SpecQuotient {
   fpair inv;
-  double inv64;
+  double inv64;   // where the pairs do not hold it
   float scale;
   bool pairs;
   __device__ __forceinline__ SpecQuotient(double a, double rhat, float s) : inv64(0.0), scale(s) {
-    fpair ap, rp;
+    fpair ap, rp, den;
     const bool in = split_double(a, ap) & split_double(rhat, rp);
-    const fpair den = pair_add(ap, rp);
-    pairs = in && well_inside(den.h);
+    pairs = pair_sum(ap, rp, den) && in;
     inv = pair_recip(den);
-    if (!pairs) slow(a + rhat);
+    if (!pairs) inv64 = spec_quotient_fp64(a + rhat, s);
   }
-  __device__ __noinline__ void slow(double den) { inv64 = (den != 0.0) ? (double)scale / den : 0.0; }
-  __device__ __forceinline__ float times(double x) const {
+  __device__ __forceinline__ float times(double x, double a, double rhat) const {
     fpair xp;
-    if (pairs && split_double(x, xp)) return pair_product(xp, inv, scale);
-    return slow_times(x);
-  }
-  __device__ __noinline__ float slow_times(double x) const {
-    if (!pairs) return (float)(x * inv64);
-    return (float)(x * ((double)inv.h + (double)inv.l) * (double)scale);
+    float out;
+    if (pairs && split_double(x, xp) && pair_product(xp, inv, scale, 1.f, out)) return out;
+    return pairs ? spec_product_fp64(x, a, rhat, scale) : (float)(x * inv64);
   }
 };
+
+// g A^-1 of the bracket A = [[a0 + r0, conj b], [b, a1 + r1]] of two coupled observed blocks: A^-1 when
+// det A > 1e-6 a11 a22, the pseudo-inverse A / tr(A)^2 of a rank-1 bracket otherwise, 0 where tr(A) = 0; rounded
+// to float.
+struct Bracket {
+  float s00, s11;
+  float2 s01;
+};
+static __device__ __noinline__ Bracket bracket_fp64(float a0, float a1, float2 b, double r0, double r1, float g) {
+  const double a = (double)a0 + r0, d = (double)a1 + r1;
+  const double br = b.x, bi = b.y;
+  const double det = a * d - (br * br + bi * bi);
+  const double tr = a + d;
+  double f = 0.0, q00 = 0.0, q11 = 0.0, q01r = 0.0, q01i = 0.0;   // A^-1 = f [[q00, q01], [conj q01, q11]]
+  if (det > 1e-6 * a * d) {
+    f = (double)g / det;
+    q00 = d; q11 = a; q01r = -br; q01i = bi;      // [[d, -conj b], [-b, a]] / det
+  } else if (tr > 0.0) {
+    f = (double)g / (tr * tr);
+    q00 = a; q11 = d; q01r = br; q01i = -bi;      // [[a, conj b], [b, d]] / tr^2
+  }
+  return {(float)(f * q00), (float)(f * q11), make_float2((float)(f * q01r), (float)(f * q01i))};
+}
+// The same in float pairs, FP64 where their error could change a result's rounding.  The determinant's relative
+// error grows with cond = a11 a22 / det, which is at most 2^10 here (up to 1e6 where it is used).
+__device__ __forceinline__ Bracket bracket(float a0, float a1, float2 b, double r0, double r1, float g) {
+  fpair p0, p1, a, d;
+  bool in = split_double(r0, p0) & split_double(r1, p1);
+  in &= pair_sum({a0, 0.f}, p0, a);
+  in &= pair_sum({a1, 0.f}, p1, d);
+  const fpair ad = pair_mul(a, d);
+  const fpair bb = pair_add(pair_mul({b.x, 0.f}, {b.x, 0.f}), pair_mul({b.y, 0.f}, {b.y, 0.f}));
+  const fpair det = pair_add(ad, {-bb.h, -bb.l});
+  const fpair f = pair_recip(det);
+  const float cond = ad.h * f.h;
+  Bracket k;
+  in &= well_inside(det.h) && a.h > 0.f && cond > 0.f && cond <= 1024.f;
+  in &= pair_product(d, f, g, cond, k.s00);
+  in &= pair_product(a, f, g, cond, k.s11);
+  in &= pair_product({-b.x, 0.f}, f, g, cond, k.s01.x);
+  in &= pair_product({b.y, 0.f}, f, g, cond, k.s01.y);
+  return in ? k : bracket_fp64(a0, a1, b, r0, r1, g);
+}
 
 }  // namespace fftenkf

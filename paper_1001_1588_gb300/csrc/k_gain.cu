@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256) gain_kernel(const GainParams p) {
     if (c < L1 && ky < p.ny) {
       const double a = ca[threadIdx.x][cl];
       bad |= !finite_double(a);
-      p.goo[i * tab + (size_t)c * p.ny + ky] = inv[q].times(a);
+      p.goo[i * tab + (size_t)c * p.ny + ky] = inv[q].times(a, a, rs[threadIdx.x][cl]);
     }
   }
   const double* xspec = p.spec + (size_t)p.n_obs * K;
@@ -71,7 +71,8 @@ __global__ void __launch_bounds__(256) gain_kernel(const GainParams p) {
       if (c < L1 && ky < p.ny) {
         const double re = cre[threadIdx.x][cl], im = cim[threadIdx.x][cl];
         bad |= !(finite_double(re) && finite_double(im));
-        p.gjo[qt * tab + (size_t)c * p.ny + ky] = make_float2(inv[q].times(re), inv[q].times(im));
+        const double a = ca[threadIdx.x][cl], r = rs[threadIdx.x][cl];
+        p.gjo[qt * tab + (size_t)c * p.ny + ky] = make_float2(inv[q].times(re, a, r), inv[q].times(im, a, r));
       }
     }
   }
@@ -199,45 +200,8 @@ cudaError_t launch_rhat_transpose(const double* rhat, double* rhat_t, int n, int
   return cudaGetLastError();
 }
 
-// g A^-1 of the bracket A = [[a0 + r0, conj b], [b, a1 + r1]], in float pairs or FP64: A^-1 when det A > 1e-6 a11 a22, the
-// pseudo-inverse A / tr(A)^2 of a rank-1 bracket otherwise, 0 where tr(A) = 0; rounded to float.
-struct Bracket {
-  float s00, s11;
-  float2 s01;
-};
-static __device__ __noinline__ Bracket bracket_fp64(float a0, float a1, float2 b, double r0, double r1, float g) {
-  const double a = (double)a0 + r0, d = (double)a1 + r1;
-  const double br = b.x, bi = b.y;
-  const double det = a * d - (br * br + bi * bi);
-  const double tr = a + d;
-  double f = 0.0, q00 = 0.0, q11 = 0.0, q01r = 0.0, q01i = 0.0;   // A^-1 = f [[q00, q01], [conj q01, q11]]
-  if (det > 1e-6 * a * d) {
-    f = (double)g / det;
-    q00 = d; q11 = a; q01r = -br; q01i = bi;      // [[d, -conj b], [-b, a]] / det
-  } else if (tr > 0.0) {
-    f = (double)g / (tr * tr);
-    q00 = a; q11 = d; q01r = br; q01i = -bi;      // [[a, conj b], [b, d]] / tr^2
-  }
-  return {(float)(f * q00), (float)(f * q11), make_float2((float)(f * q01r), (float)(f * q01i))};
-}
-// The same in float pairs (48 bits; the determinant keeps at least 28 of them where it is used, since
-// it is above 1e-6 of the product of the diagonal).
-__device__ __forceinline__ Bracket bracket(float a0, float a1, float2 b, double r0, double r1, float g) {
-  fpair p0, p1;
-  const bool in = split_double(r0, p0) & split_double(r1, p1);
-  const fpair a = pair_add({a0, 0.f}, p0), d = pair_add({a1, 0.f}, p1);
-  const fpair ad = pair_mul(a, d);
-  const fpair bb = pair_add(pair_mul({b.x, 0.f}, {b.x, 0.f}), pair_mul({b.y, 0.f}, {b.y, 0.f}));
-  const fpair det = pair_add(ad, {-bb.h, -bb.l});
-  if (!in || !(det.h > 2e-6f * ad.h) || !well_inside(det.h) || !well_inside(a.h) || !well_inside(d.h))
-    return bracket_fp64(a0, a1, b, r0, r1, g);   // (nearly) singular, or out of the pairs' range
-  const fpair f = pair_recip(det);
-  return {pair_product(f, d, g), pair_product(f, a, g),
-          make_float2(pair_product(f, {-b.x, 0.f}, g), pair_product(f, {b.y, 0.f}, g))};
-}
-
 // One thread per wavenumber (column-major index at = k_x ny + k_y).  The bracket A = chat_OO +
-// diag(rhat) is inverted (bracket above; in FP64 the kernel took 465 us at 4096^2 with three blocks),
+// diag(rhat) is inverted (bracket, dd.cuh; in FP64 the kernel took 465 us at 4096^2 with three blocks),
 // scaled by 1/(ny nx) and rounded to float, and K_r = chat_{r,O} A^-1 is formed in FP32.
 __global__ void __launch_bounds__(256) coupled_gain_kernel(const CoupledGainParams p) {
   const size_t tab = (size_t)(p.L + 1) * p.ny;
@@ -250,9 +214,7 @@ __global__ void __launch_bounds__(256) coupled_gain_kernel(const CoupledGainPara
     float s00 = 0.f, s11 = 0.f;
     float2 s01 = make_float2(0.f, 0.f);
     if (p.n_obs == 1) {
-      const double r = p.rhat_t[at];
-      float den;
-      s00 = denominator(a0, r, den) ? __fdiv_rn(p.inv_G, den) : (float)quotient_fp64(a0, r, p.inv_G);
+      s00 = quotient(a0, p.rhat_t[at], p.inv_G);
     } else {
       const Bracket k = bracket(a0, a1, b10, p.rhat_t[at], p.rhat_t[tab + at], p.inv_G);
       s00 = k.s00;

@@ -215,11 +215,11 @@ __device__ __forceinline__ bool split_gains(const SplitParams& p, const SplitIte
         const double a = p.spec[(size_t)i * tab + at];
         ok &= finite_double(a);
         const SpecQuotient q(a, rr, p.inv_G);
-        acc[i * NY + ky] = q.times(a);
+        acc[i * NY + ky] = q.times(a, a, rr);
         for (int u = 0; u < n_un; ++u) {
           const double* s = p.spec + (size_t)p.n_obs * tab + 2 * ((size_t)(i * n_un + u) * tab + at);
           ok &= finite_double(s[0]) && finite_double(s[1]);
-          x0[(size_t)u * NY] = make_float2(q.times(s[0]), q.times(s[1]));
+          x0[(size_t)u * NY] = make_float2(q.times(s[0], a, rr), q.times(s[1], a, rr));
         }
         continue;
       }

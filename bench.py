@@ -154,11 +154,19 @@ def cufft_reference(ny, nx, M_, N_, n_obs, dev, steps=3, chunk=20):
 def pick_fused_schedule(plan, step, stream, reps=2):
     """Autotune the fused column pass's line-FFT schedule (0: 16 values per thread, 1: 8 values,
     twice the threads) on the workload itself, before the warm-up: each candidate runs `reps`
-    analyses after one untimed one; the faster is kept.  Returns the chosen schedule."""
+    analyses after one untimed one; the faster is kept.  Returns the chosen schedule.  Where the
+    plan does not run the fused pass (small grids, whose columns read rhat as it is, and shapes
+    with separate column passes) there is nothing to choose: the default stays."""
     import torch
     from paper_1001_1588_gb300 import abi
     fused = abi.fftenkf_pass_count() - 1
     base = abi.fftenkf_get_schedule(plan.handle)
+    abi.fftenkf_set_profiling(plan.handle, True)
+    step()
+    ran = abi.fftenkf_pass_times(plan.handle)
+    abi.fftenkf_set_profiling(plan.handle, False)
+    if not (ran["col_fused"][1] and ran["rhat_transpose"][1]):
+        return base[fused]
     best, best_ms = base[fused], None
     for sel in (0, 1):
         sched = list(base)

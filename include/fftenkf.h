@@ -188,7 +188,11 @@ fftenkf_status fftenkf_set_expire_first_wait(fftenkf_plan plan, int on);
  * last read (or enable), and resets the totals.  Passes are numbered
  * 0..fftenkf_pass_count()-1 and named by fftenkf_pass_name.  Pass 0 ("mean")
  * is retired (the anomaly rows take the first member as pivot): it keeps its
- * number so that the others keep theirs, and always reports 0 launches. */
+ * number so that the others keep theirs, and always reports 0 launches.
+ * On small grids and ensembles one launch does the work of several passes: rows
+ * of anomalies and innovations together report as "row_fwd_anomaly", columns
+ * that form statistics, gains and update together as "col_fused" (and then no
+ * "rhat_transpose" or "gain"). */
 fftenkf_status fftenkf_set_profiling(fftenkf_plan plan, int enable);
 fftenkf_status fftenkf_pass_times(fftenkf_plan plan, double* total_ms, int* launches, int n_passes);
 int fftenkf_pass_count(void);
@@ -202,7 +206,11 @@ const char* fftenkf_pass_name(int pass);
  * on one SM.  set returns EINVAL for out-of-range entries and EUNSUPPORTED if a
  * choice does not fit
  * in shared memory; the plan keeps its previous schedule then.  The schedule
- * changes speed only: every schedule computes the same analysis. */
+ * changes speed only: every schedule computes the same analysis.
+ * With 0 for every pass with transforms (the default) the library may use, on
+ * small grids and ensembles, launches of its own plans in place of the passes
+ * (see fftenkf_set_profiling).  Any other entry of such a pass selects the passes
+ * for the whole plan, each with the plan of its entry. */
 fftenkf_status fftenkf_set_schedule(fftenkf_plan plan, const int* sched, int n);
 fftenkf_status fftenkf_get_schedule(fftenkf_plan plan, int* sched, int n);
 

@@ -294,8 +294,8 @@ static fftenkf_status get_workspace(fftenkf_plan p, void* ws, char** out) {
 //   inverse rows: up to 2^23 points of the ensemble and 2048-point rows (1024^2 N=5 25 -> 21, but N=20 65 -> 72)
 enum SplitBits { kSplitRows = 1, kSplitCols = 2, kSplitInv = 4 };
 static int split_rule(fftenkf_plan p) {
-  for (int a = 0; a < kPassCount; ++a)
-    if (p->sched[a] != 0) return 0;   // a schedule was chosen: the passes it names
+  for (int a : {kPassRowAnom, kPassStats, kPassRowInnov, kPassUpdate, kPassRowInv, kPassFused})
+    if (p->sched[a] != 0) return 0;   // a schedule was chosen for a pass with transforms: the passes it names
   int bits = 0;
   if (p->expire_first_wait == 0 && split_rows_supported(p->L) && (p->L <= 1024 || 2 * p->M * (p->ny / 8) <= sm_count()))
     bits |= kSplitRows;

@@ -129,29 +129,47 @@ __device__ __forceinline__ float quotient(float val, double rhat, float inv_G) {
 static __device__ __noinline__ double spec_quotient_fp64(double den, float scale) {
   return (den != 0.0) ? (double)scale / den : 0.0;
 }
-static __device__ __noinline__ float spec_product_fp64(double x, double a, double rhat, float scale) {
-  return (float)(x * spec_quotient_fp64(a + rhat, scale));
-}
+__device__ __forceinline__ int exponent_of(double x) { return (int)((uint32_t)__double2hiint(x) >> 20) & 0x7ff; }
 
 // scale / (a + rhat) for a caller's spectrum, and its products with entries x of the spectrum, each rounded
-// to float once
+// to float once.  Steep spectra (a squared-exponential one over most of the plane) hold entries below 2^-74:
+// as a or rhat they count as 0 beside a sum of at least 2^-24 (2^-50 of it), as x their exponent is raised by
+// 96 and the result lowered again.  (In FP64 such entries took the gain kernel 1.3 to 3 times as long: 512^2,
+// one observed of three blocks, 26 us instead of 9; 12.5 us with FP64 throughout.)
 struct SpecQuotient {
   fpair inv;
-  double inv64;   // where the pairs do not hold it
+  double inv64;   // formed where the pairs do not hold it, or at the first product that needs it
   float scale;
-  bool pairs;
+  bool pairs, formed;
   __device__ __forceinline__ SpecQuotient(double a, double rhat, float s) : inv64(0.0), scale(s) {
     fpair ap, rp, den;
-    const bool in = split_double(a, ap) & split_double(rhat, rp);
-    pairs = pair_sum(ap, rp, den) && in;
+    const bool ta = exponent_of(a) < 949, tr = exponent_of(rhat) < 949;
+    const bool in = (split_double(ta ? 0.0 : a, ap) & split_double(tr ? 0.0 : rhat, rp));
+    pairs = pair_sum(ap, rp, den) && in && (!(ta | tr) || fabsf(den.h) >= 0x1p-24f);
     inv = pair_recip(den);
+    formed = !pairs;
     if (!pairs) inv64 = spec_quotient_fp64(a + rhat, s);
   }
-  __device__ __forceinline__ float times(double x, double a, double rhat) const {
+  __device__ __forceinline__ float times(double x, double a, double rhat) {
+    if (!pairs) return (float)(x * inv64);
+    const int e = exponent_of(x);
+    const bool low = e < 949;
     fpair xp;
     float out;
-    if (pairs && split_double(x, xp) && pair_product(xp, inv, scale, 1.f, out)) return out;
-    return pairs ? spec_product_fp64(x, a, rhat, scale) : (float)(x * inv64);
+    // (zeros, subnormals and exponents below 853 stay out of split_double's range when raised)
+    const bool in = split_double(low ? __hiloint2double(__double2hiint(x) + (96 << 20), __double2loint(x)) : x, xp);
+    const bool ok = pair_product(xp, inv, scale, 1.f, out);
+    if (!low) {
+      if (in && ok) return out;
+    } else if (e < 853) {   // below 2^-170
+      if (fabsf(inv.h) * scale < 0x1p18f) return 0.f;
+    } else if (in) {
+      if (fabsf(xp.h * inv.h * scale) < 0x1p-58f) return 0.f;   // below 2^-154
+      if (ok && fabsf(out) >= 0x1p-30f) return out * 0x1p-96f;   // exact: a normal float
+    }
+    if (!formed) inv64 = spec_quotient_fp64(a + rhat, scale);
+    formed = true;
+    return (float)(x * inv64);
   }
 };
 

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) gain_kernel(const GainParams p) {
     const int cl = threadIdx.y + 8 * q;
     return SpecQuotient(ca[threadIdx.x][cl], rs[threadIdx.x][cl], p.scale);
   };
-  const SpecQuotient inv[TB / 8] = {quotient(0), quotient(1), quotient(2), quotient(3)};
+  SpecQuotient inv[TB / 8] = {quotient(0), quotient(1), quotient(2), quotient(3)};
 #pragma unroll
   for (int q = 0; q < TB / 8; ++q) {
     const int cl = threadIdx.y + 8 * q;

@@ -214,7 +214,7 @@ __device__ __forceinline__ bool split_gains(const SplitParams& p, const SplitIte
         const size_t at = (size_t)ky * (p.L + 1) + c;
         const double a = p.spec[(size_t)i * tab + at];
         ok &= finite_double(a);
-        const SpecQuotient q(a, rr, p.inv_G);
+        SpecQuotient q(a, rr, p.inv_G);
         acc[i * NY + ky] = q.times(a, a, rr);
         for (int u = 0; u < n_un; ++u) {
           const double* s = p.spec + (size_t)p.n_obs * tab + 2 * ((size_t)(i * n_un + u) * tab + at);

@@ -19,6 +19,7 @@
 #include <string>
 
 #include "../../include/fftenkf.h"
+#include "morph_rule.cuh"
 
 namespace fftenkf {
 void set_last_error(const std::string& msg);
@@ -26,7 +27,7 @@ void set_last_error(const std::string& msg);
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = fftenkf::kMorphThreads;
 constexpr float kMaxOffset = 4194304.f;  // 2^22 cells: offsets are clamped to this for indexing
 constexpr int kMaxIter = 1024;
 
@@ -81,7 +82,7 @@ __device__ __forceinline__ float interp(const float* __restrict__ f, const Stenc
 // displacements of up to 3 cells: 2530 us (a thread per node gathering 8 words from global memory per step,
 // bound by issue), 1854 with staged blocks, 1377 like this.  The inverse transform, one gather a node, is
 // faster without tiles (129 us against 222, K = 4).
-constexpr int kTX = 64, kHalo = 6, kRW = kTX + 2 * kHalo;
+constexpr int kTX = fftenkf::kMorphTX, kHalo = 6, kRW = kTX + 2 * kHalo;
 template <int TY>
 struct Tile {
   float2 v[TY + 2 * kHalo][kRW];
@@ -328,17 +329,13 @@ extern "C" fftenkf_status fftenkf_morph_forward(const float* u, const float* u_r
   if (overlaps(r, r_bytes, u, r_bytes) || overlaps(r, r_bytes, u_ref, (size_t)n_blocks * plane) ||
       overlaps(r, r_bytes, ext, (size_t)2 * n_members * plane))
     return mfail(FFTENKF_EINVAL, std::string(who) + ": the residual blocks of ext overlap an input");
-  const int tiles_x = (nx + kTX - 1) / kTX;
+  const int tiles_x = nx / kTX + (nx % kTX != 0);
   cudaStream_t st_ = static_cast<cudaStream_t>(stream);
-  // Tiles of 16 rows from one wave of 8 CTAs per SM on; 8 rows below (256^2, K = 4: 15 us, 17 with 16 rows);
-  // no tiles where they hardly pay their halo and padding: up to three CTAs of nodes per SM (62 x 173, K = 9:
-  // 11 us, 13 with tiles), or less than 60 % of the tiles' columns on the grid (2400 x 65, K = 6: 40 us, 42
-  // with tiles; 1692 x 77, 60 %: 35.5 both).
-  const long long sms = sm_of_current(), tiles16 = (long long)tiles_x * ((ny + 15) / 16) * n_members;
-  if ((long long)ny * nx * n_members <= 3 * sms * kThreads || 5 * nx < 3 * kTX * tiles_x)
+  const fftenkf::MorphForm form = fftenkf::morph_form(ny, nx, n_members, sm_of_current());
+  if (form == fftenkf::kMorphGather)
     morph_forward_gather<<<member_grid(ny * nx, n_members, resident_ctas(morph_forward_gather)), kThreads, 0, st_>>>(
         u, u_ref, ext, n_blocks, n_members, ny, nx, n_iter, tol);
-  else if (tiles16 >= 8 * sms)
+  else if (form == fftenkf::kMorphTiles16)
     morph_forward_kernel<16, 8><<<dim3((unsigned)(tiles_x * ((ny + 15) / 16)), (unsigned)n_members), kThreads, 0, st_>>>(
         u, u_ref, ext, n_blocks, n_members, ny, nx, n_iter, tol, tiles_x);
   else

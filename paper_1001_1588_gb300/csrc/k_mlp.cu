@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(256) mlp_max_kernel(const MlpBinParams p) {
   __shared__ float red8[8];
   const double* c = p.chat + (size_t)blockIdx.y * p.bins.K1;
   stream_order_wait();
+  next_may_start();
   float mx = 0.f;
 #pragma unroll 4
   for (int i = blockIdx.x * 256 + threadIdx.x; i < p.bins.K1; i += gridDim.x * 256) mx = fmaxf(mx, to_float(c[i]));
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(256) mlp_binsum_kernel(const MlpBinParams p) {
 #pragma unroll
   for (int e = 0; e < E; ++e) at[e] = i0 + threadIdx.x + 256 * e < i1 ? __ldg(p.bins.order + i0 + threadIdx.x + 256 * e) : ~0u;
   stream_order_wait();
+  next_may_start();
   const double* c = p.chat + (size_t)blockIdx.y * p.bins.K1;
   float v[E];
 #pragma unroll
@@ -148,6 +150,7 @@ __global__ void __launch_bounds__(kBins) mlp_binfin_kernel(const MlpBinParams p)
   __shared__ float red4[kBins / 32];
   __shared__ float cm;
   stream_order_wait();
+  next_may_start();
   const int smp = blockIdx.x;
   const float mu = bin_features(p.bins, smp, p.feat + (size_t)smp * kIn, red4, &cm);
   if (threadIdx.x == 0) p.mean[smp] = mu;
@@ -166,6 +169,7 @@ struct MlpUnbinParams {
 __global__ void __launch_bounds__(256) mlp_unbin_kernel(const MlpUnbinParams p) {
   const int K1 = p.ny * (p.L + 1);
   stream_order_wait();
+  next_may_start();
   const bool plain = *p.flag != 0;
   for (int i = blockIdx.x * 256 + threadIdx.x; i < K1; i += gridDim.x * 256) {
     if (plain) {
@@ -315,6 +319,7 @@ __global__ void __launch_bounds__(32 * NW) mlp_fwd_kernel(const MlpFwdParams p) 
   const int s0 = blockIdx.x * S, nsamp = min(S, p.B - s0);
   const bool vec = (reinterpret_cast<uintptr_t>(p.params) & 15) == 0;
   stream_order_wait();
+  next_may_start();
   load_samples<S>(a, p.X, s0, nsamp, 32 * NW);
   mlp_forward<S, NW>(a, p.params, vec, threadIdx.x >> 5, threadIdx.x & 31);
   for (int i = threadIdx.x; i < nsamp * kOut; i += 32 * NW) p.out[(size_t)s0 * kOut + i] = a.out[i / kOut][i % kOut];
@@ -330,6 +335,7 @@ struct MlpGradParams {
 };
 __global__ void __launch_bounds__(256) mlp_zero_kernel(const MlpGradParams p) {
   stream_order_wait();
+  next_may_start();
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i < kParams) p.grads[i] = 0.f;
   if (i == 0) *p.loss = 0.f;
@@ -406,6 +412,7 @@ __global__ void __launch_bounds__(256) mlp_bwd_kernel(const MlpGradParams p) {
   const bool vec = (reinterpret_cast<uintptr_t>(p.params) & 15) == 0;
   const bool gvec = (reinterpret_cast<uintptr_t>(p.grads) & 15) == 0;
   stream_order_wait();
+  next_may_start();
   load_samples<S>(a, p.X, s0, nsamp, 256);
   mlp_forward<S, 8>(a, p.params, vec, tid >> 5, tid & 31);
   const float scale = 2.f / ((float)p.B * kOut);
@@ -434,6 +441,7 @@ struct MlpAdamParams {
 };
 __global__ void __launch_bounds__(256) mlp_adam_kernel(const MlpAdamParams p) {
   stream_order_wait();
+  next_may_start();
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= kParams) return;
   const float gi = p.g[i];
@@ -461,6 +469,7 @@ __global__ void __launch_bounds__(1024) mlp_head_kernel(const MlpHeadParams p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool vec = (reinterpret_cast<uintptr_t>(p.params) & 15) == 0;
   stream_order_wait();
+  next_may_start();
   const float mu = bin_features(p.bins, 0, &a.x[0][0], red4, &cm);
   mlp_forward<1, 32>(a, p.params, vec, warp, lane);
   bool bad = false;

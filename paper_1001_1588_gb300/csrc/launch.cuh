@@ -16,10 +16,15 @@ cudaError_t kernel_shape(const void* kern, int threads, size_t smem, int* per_sm
 // finished and its writes are visible; nothing of an earlier kernel is read or overwritten before it.
 // Data of earlier kernels is read by plain loads: the compiler may move __ldg and loads through const
 // __restrict__ pointers, which it takes for loads of constants, ahead of this wait.
-// It then lets the next kernel of the stream be brought onto SMs that have room, where it waits here.
-__device__ __forceinline__ void stream_order_wait() {
-  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
-}
+__device__ __forceinline__ void stream_order_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Lets the next kernel of the stream be brought onto SMs that have room, where it waits in stream_order_wait(),
+// once every CTA of this one has called it or left (without it: once every CTA has left).  For kernels that leave
+// the SM's on-chip memory alone, as the network's.  The split and sine passes do without: the next pass's waiting
+// CTAs hold shared memory, which is then missing as first-level cache for spills and instructions of the pass that
+// runs (called at the start of each: 48 x 128, N = 25, 2 of 4 blocks observed 66 us, 34 without; 1024 x 48, N = 25,
+// 4 blocks 346 and 259; 64^2 14 us both; called before a CTA's last stores: 35, 270, 14).
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Launch with the stream's order kept by stream_order_wait() at the kernel's start: the launch latency
 // of a kernel overlaps the one before it (2-3 us between dependent kernels otherwise).

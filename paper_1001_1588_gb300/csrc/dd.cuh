@@ -166,6 +166,10 @@ struct SpecQuotient {
     } else if (in) {
       if (fabsf(xp.h * inv.h * scale) < 0x1p-58f) return 0.f;   // below 2^-154
       if (ok && fabsf(out) >= 0x1p-30f) return out * 0x1p-96f;   // exact: a normal float
+      // a subnormal float: out, rounded already, is rounded again to a multiple of 2^-149 (in this scale 2^-53),
+      // which is wrong only where it lies half-way
+      const float z = fabsf(out) * 0x1p53f, k = rintf(z);
+      if (ok && fabsf(z - k) != 0.5f) return copysignf(__uint_as_float((uint32_t)k), out);
     }
     if (!formed) inv64 = spec_quotient_fp64(a + rhat, scale);
     formed = true;

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(256) coupled_gain_kernel(const CoupledGainPara
 cudaError_t launch_coupled_gain(const CoupledGainParams& p, cudaStream_t s) {
   const size_t tab = (size_t)(p.L + 1) * p.ny;
   long long blocks = (long long)((tab + 255) / 256);
-  if (blocks > 152LL * 8) blocks = 152LL * 8;
+  if (blocks > 8LL * sm_count()) blocks = 8LL * sm_count();
   coupled_gain_kernel<<<(unsigned)blocks, 256, 0, s>>>(p);
   return cudaGetLastError();
 }

@@ -22,7 +22,7 @@ int sine_col_groups(int ny, int nx, int n_obs, int M, int N) {
     const int by_threads = sine_col_threads(n_obs) / ((g * T + 31) / 32 * 32);
     if (per_sm > by_threads) per_sm = by_threads;
     if (per_sm < 1) per_sm = 1;
-    const long long slots = 152 * per_sm, cost = ((N + g - 1) / g) * (((nx - 1) / 2 + slots - 1) / slots);
+    const long long slots = sm_count() * per_sm, cost = ((N + g - 1) / g) * (((nx - 1) / 2 + slots - 1) / slots);
     if (best == 0 || cost < best_cost) {
       best = g;
       best_cost = cost;

@@ -371,8 +371,7 @@ inline cudaError_t launch_sine_rows(K kern, int P, const SineParams& p, int unit
   if (lpc < 1) return cudaErrorInvalidConfiguration;
   lpc = lpc >= sine_tile_lines(P) ? sine_tile_lines(P) : lpc >= 2 ? 2 : 1;
   const size_t smem = (size_t)sine_tile_lines(P) * row_pitch(P) * sizeof(float2);
-  int per_sm = 0;
-  cudaError_t e = kernel_shape(reinterpret_cast<const void*>(kern), T * lpc, smem, &per_sm);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   return launch_overlapped(kern, dim3((unsigned)units), T * lpc, smem, s, p);
 }
@@ -391,8 +390,7 @@ inline cudaError_t sine_cols_P(const SineParams& p, cudaStream_t s) {
   const size_t smem = (size_t)p.acc_bytes + (size_t)p.groups * col_line_slots(P) * sizeof(float2);
   const int threads = P / plan_V(P, 0) * p.groups;
   auto kern = sine_cols_kernel<P, NOBS>;
-  int per_sm = 0;
-  cudaError_t e = kernel_shape(reinterpret_cast<const void*>(kern), threads, smem, &per_sm);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   return launch_overlapped(kern, dim3((unsigned)((p.nx - 1) / 2)), threads, smem, s, p);
 }

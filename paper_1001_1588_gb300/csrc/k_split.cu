@@ -2,39 +2,24 @@
 // storage type or observed-block count).
 #include <map>
 #include <mutex>
-#include <tuple>
+#include <utility>
 
 #include "k_split.cuh"
 
 namespace fftenkf {
 
-cudaError_t kernel_shape(const void* kern, int threads, size_t smem, int* per_sm) {
+cudaError_t allow_smem(const void* kern, size_t smem) {
   static std::mutex mu;
-  static std::map<std::tuple<int, const void*, int, size_t>, int> known;
   static std::map<std::pair<int, const void*>, size_t> allowed;   // largest request so far: never lowered
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
-  const auto key = std::make_tuple(dev, kern, threads, smem);
-  const auto it = known.find(key);
-  if (it != known.end()) {
-    *per_sm = it->second;
-    return cudaSuccess;
-  }
   size_t& a = allowed[std::make_pair(dev, kern)];
-  if (smem > a) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    a = smem;
-  }
-  int n = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem);
-  if (e != cudaSuccess) return e;
-  if (n < 1) n = 1;
-  known[key] = n;
-  *per_sm = n;
-  return cudaSuccess;
+  if (smem <= a) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) a = smem;
+  return e;
 }
 
 bool split_rows_supported(int L) { return row_line_supported(L); }

@@ -451,8 +451,7 @@ inline cudaError_t launch_rows_split(K kern, int L, int V, SplitParams p, int un
   if (lpc < 1) lpc = 1;
   if (lpc > p.R) lpc = p.R;
   const size_t smem = (size_t)p.R * row_pitch(L) * sizeof(float2);
-  int per_sm = 0;
-  cudaError_t e = kernel_shape(reinterpret_cast<const void*>(kern), T * lpc, smem, &per_sm);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   return launch_overlapped(kern, dim3((unsigned)units), T * lpc, smem, st, p);
 }
@@ -488,8 +487,7 @@ inline cudaError_t col_split_NY(const SplitParams& p, int units, cudaStream_t st
   constexpr int V = plan_V(NY, split_col_sel(NY, CROSS)), T = NY / V;
   const size_t smem = (size_t)p.acc_bytes + (size_t)p.groups * col_line_slots(NY) * sizeof(float2);
   auto kern = col_split_kernel<NY, V, NOBS, CROSS, DRAWN>;
-  int per_sm = 0;
-  cudaError_t e = kernel_shape(reinterpret_cast<const void*>(kern), T * p.groups, smem, &per_sm);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   return launch_overlapped(kern, dim3((unsigned)units), T * p.groups, smem, st, p);
 }

@@ -1,16 +1,14 @@
-// Kernel launches of the analysis passes: shape look-ups made once per (device, kernel, shape), and
-// launches that may overlap the tail of the kernel before them (programmatic dependent launch).
+// Kernel launches of the analysis passes: dynamic shared memory allowed once per (device, kernel), and
+// launches whose latency overlaps the kernel before them (programmatic dependent launch).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace fftenkf {
 
-// Resident CTAs per SM of `kern` with `threads` and `smem` bytes of dynamic shared memory, after
-// allowing it that much.  The attribute call and the occupancy query cost several microseconds of host
-// time, more than a launch, so the answers are kept, one entry per (device, kernel, threads, smem)
-// that was ever launched.
-cudaError_t kernel_shape(const void* kern, int threads, size_t smem, int* per_sm);
+// Allows `kern` `smem` bytes of dynamic shared memory on the current device.  The attribute call costs
+// more host time than a launch, so it is made once per (device, kernel) and larger request.
+cudaError_t allow_smem(const void* kern, size_t smem);
 
 // In a kernel launched with launch_overlapped: returns once every earlier kernel of the stream has
 // finished and its writes are visible; nothing of an earlier kernel is read or overwritten before it.

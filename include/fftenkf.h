@@ -256,9 +256,10 @@ fftenkf_status fftenkf_analyze_batched(fftenkf_batch batch, void* const* ensembl
                                        const void* const* perturbations, const double* const* rhat,
                                        void* workspace, void* stream);
 /* Autotuner: times every candidate CTA size (128, 256 threads) of the forward
- * rows, columns and inverse rows on zero-filled scratch inputs of the batch's
- * shapes (allocated for the call: one copy of every item's inputs) and keeps
- * the fastest; best_ms (may be NULL) receives the sum of the best pass times. */
+ * rows, columns and inverse rows on scratch inputs of the batch's shapes (zero
+ * fields and a positive rhat, allocated for the call: one copy of every item's
+ * inputs), the shapes one after another on `stream`, and keeps the fastest;
+ * best_ms (may be NULL) receives the sum of the best pass times. */
 fftenkf_status fftenkf_batch_autotune(fftenkf_batch batch, void* workspace, void* stream, double* best_ms);
 /* Chosen CTA size and schedule of each batched pass (7 passes: mean, anomaly
  * rows, statistics, gain, innovation rows, update, inverse rows; passes that share

@@ -342,8 +342,9 @@ extern "C" fftenkf_status fftenkf_analyze_batched(fftenkf_batch b, void* const* 
   return FFTENKF_OK;
 }
 
-// Time the CTA sizes of every stage on zero-filled scratch inputs of the batch's shapes and keep the
-// fastest.  Allocates the scratch inputs (one ensemble's worth per item) for the duration of the call.
+// Time the CTA sizes of every stage on scratch inputs of the batch's shapes, the classes one after another, and
+// keep the fastest.  The fields are zero; rhat is positive (the byte 0x3f repeated, 4.8e-4): with rhat = 0 every
+// denominator would vanish and take the column pass's FP64 branch, which real inputs do not.  Allocates the scratch inputs (one ensemble's worth per item) for the duration of the call.
 extern "C" fftenkf_status fftenkf_batch_autotune(fftenkf_batch b, void* workspace, void* stream, double* best_ms) {
   set_last_error("");
   if (!b) return bfail(FFTENKF_EINVAL, "null argument");
@@ -360,11 +361,16 @@ extern "C" fftenkf_status fftenkf_batch_autotune(fftenkf_batch b, void* workspac
     oe[i] = bytes; bytes = rup(bytes + d.n_members * G * es, 256);
     od[i] = bytes; bytes = rup(bytes + G * 4, 256);
     op[i] = bytes; bytes = rup(bytes + d.n_members * G * es, 256);
-    orh[i] = bytes; bytes = rup(bytes + (size_t)d.ny * (d.nx / 2 + 1) * 8, 256);
+  }
+  const size_t field_bytes = bytes;
+  for (int i = 0; i < b->count; ++i) {
+    orh[i] = bytes;
+    bytes = rup(bytes + (size_t)b->dims[i].ny * (b->dims[i].nx / 2 + 1) * 8, 256);
   }
   char* scratch = nullptr;
   if (cudaMalloc(&scratch, bytes) != cudaSuccess) return bfail(FFTENKF_ENOMEM, "autotune scratch allocation failed");
-  cudaMemsetAsync(scratch, 0, bytes, s);
+  cudaMemsetAsync(scratch, 0, field_bytes, s);
+  cudaMemsetAsync(scratch + field_bytes, 0x3f, bytes - field_bytes, s);
   std::vector<void*> ens(b->count), pert(b->count);
   std::vector<const float*> dat(b->count);
   std::vector<const double*> rh(b->count);

@@ -35,8 +35,8 @@ PASSES = [
     (re.compile(r"col_update_kernel"), "col_update"),
     (re.compile(r"row_inv_kernel"), "row_inv"),
 ]
-OURS = re.compile(r"(rhat_transpose|row_anom|row_fwd|col_fused|col_stats|col_update|row_inv|gain_kernel|"
-                  r"coupled_gain|chat_out|odd_extend|interior_copy|rhat_extend|sine_tables|mlp_|morph|batch|"
+OURS = re.compile(r"(rhat_transpose|row_anom|row_fwd|row_split|col_split|col_fused|col_stats|col_update|row_inv|gain_kernel|"
+                  r"coupled_gain|chat_out|odd_extend|interior_copy|rhat_extend|sine_|mlp_|morph|"
                   r"stage_twiddles|plain_twiddles)")
 
 

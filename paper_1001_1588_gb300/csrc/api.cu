@@ -282,28 +282,59 @@ static fftenkf_status get_workspace(fftenkf_plan p, void* ws, char** out) {
 }
 
 // Which passes of a call run split into independent CTAs (k_split.cuh): bit 0 the forward rows, bit 1
-// the columns, bit 2 the inverse rows.  Measured on a 152-SM GB300 (us, pipelined passes -> split):
+// the columns, bit 2 the inverse rows.  The lines lie where both sides, measured on a 152-SM GB300 over 3700 shapes
+// (columns of 32 to 4096 points, rows of 48 to 4096, 3 to 25 members, up to four blocks, FP32 and BF16), cross; us,
+// pipelined -> split:
 //   rows: 64^2 N=5 27 -> 8, 512^2 N=20 71 -> 34, 1536x768 N=25 3 blocks 382 -> 259, 2048^2 N=20 4 blocks
 //     1088 -> 1025; rows of 4096 points only where the pipelined pass has fewer tiles of 8 rows than half
-//     the SMs (256x4096 N=4 66 -> 39, but 512x4096 N=20 4 blocks 597 -> 841)
-//   columns: up to 768 points always (512^2 N=5 3 blocks 101 -> 30, 512x4096 N=20 4 blocks 683 -> 598);
-//     above, with one observed and no other block (1024^2 N=20 163 -> 100, 2048^2 N=10 352 -> 213), with all
-//     blocks observed at 1024 (186 -> 187, two launches fewer), where the fused pass does not apply for the
-//     observed blocks (1024x2048 N=15, 3 of 4 observed 851 -> 672), and where the fused pass would leave
-//     more than half its column groups idle (1024x512 N=8 167 -> 104, but 1024^2 N=20 192 -> 218)
+//     the SMs (256x4096 N=4 66 -> 39, but 512x4096 N=20 4 blocks 597 -> 841); FP32 rows of 384 points (24 values on
+//     each of 8 threads) not with many members on long columns (estimate of 1536x384 N=25 3 blocks 343 -> 415,
+//     3072x384 615 -> 692; but 2048x384 536 -> 498, and BF16 of 1536x384 551 -> 371)
+//   columns: up to 768 points always (512^2 N=5 3 blocks 101 -> 30, 512x4096 N=20 4 blocks 683 -> 598); above, with one observed and no other block (1024^2 N=20 163 -> 100, 2048^2
+//     N=10 352 -> 213), with all blocks observed at 1024 (186 -> 187, two launches fewer; but not for few members
+//     on long rows, 1024x2048 N=3 4 blocks 438 -> 517, 1024x4096 N=3 2 blocks 348 -> 387), where the fused pass does
+//     not apply for the observed blocks (1024x2048 N=15, 3 of 4 observed 851 -> 672), and where the fused pass would
+//     leave more than half its column groups idle (1024x512 N=8 167 -> 104, but 1024^2 N=20 192 -> 218)
 //   inverse rows: up to 2^23 points of the ensemble and 2048-point rows (1024^2 N=5 25 -> 21, but N=20 65 -> 72)
 enum SplitBits { kSplitRows = 1, kSplitCols = 2, kSplitInv = 4 };
-static int split_rule(fftenkf_plan p) {
+// what a call's columns do: sums, gains and update; the sums alone; the update with gains of a caller's spectrum
+enum ColumnWork { kEstimateAndUpdate, kEstimateOnly, kUpdateOnly };
+
+// Columns of an update with a caller's spectrum.  Without sums the pipelined update spreads every member over
+// the chip, the split columns keep a column's members on one CTA: these pay (no separate gain pass) for short
+// columns, and for longer ones where the grid has enough of them for its members.  us, pipelined -> split columns:
+// 64^2 N=3 44 -> 17, 1024^2 N=3 48 -> 45, but 512x48 N=25 1 of 3 observed 40 -> 43, 768x48 N=25 4 blocks 105 -> 237,
+// 1024x48 N=25 2 of 4 observed 74 -> 137, 192^2 N=3 all of 3 observed 37 -> 56 (that instantiation spills).
+static bool split_update_columns(fftenkf_plan p) {
+  const int ny = p->ny, nx = p->nx, N = p->N, n = p->n_obs;
+  const bool others = p->n_un > 0, many = nx >= 512 && N >= 8;
+  if (ny <= 128) return true;
+  if (ny <= 256) return n <= 2 || others || many;
+  if (ny <= 512) return n == 1 ? (ny == 384 || nx >= 4 * N) : (nx >= 6 * N && (others || ny == 512 || many));
+  if (ny == 768) return n == 1 ? (nx >= 6 * N && (!others || nx < 1024)) : (n > 2 && many);
+  if (ny == 1024) return (!others && n <= 2 && nx >= 8 * N) || ((n == 2 || n == 3) && many);
+  return false;
+}
+
+static int split_rule(fftenkf_plan p, ColumnWork work) {
   for (int a : {kPassRowAnom, kPassStats, kPassRowInnov, kPassUpdate, kPassRowInv, kPassFused})
     if (p->sched[a] != 0) return 0;   // a schedule was chosen for a pass with transforms: the passes it names
   int bits = 0;
-  if (p->expire_first_wait == 0 && split_rows_supported(p->L) && (p->L <= 1024 || 2 * p->M * (p->ny / 8) <= sm_count()))
+  const bool wide_f32 = p->storage == FFTENKF_F32 && p->L == 192 && p->N >= 16 && p->ny >= 1536 && p->ny != 2048;
+  if (p->expire_first_wait == 0 && split_rows_supported(p->L) && !wide_f32 &&
+      (p->L <= 1024 || 2 * p->M * (p->ny / 8) <= sm_count()))
     bits |= kSplitRows;
   if (!p->coupled && split_cols_supported(p->ny, p->n_obs, p->M)) {
-    const bool all = p->n_un == 0;
-    if (p->ny <= 768 || (p->ny == 1024 && all) || p->M == 1 || (p->ny == 1024 && p->n_obs > 2) ||
-        (p->use_fused() && 2 * (p->L + 1) <= col_fused_groups(p->ny, 0)))
-      bits |= kSplitCols;
+    const bool all = p->n_un == 0, few_long = p->N < 8 && p->nx >= 2048;
+    bool cols = p->ny <= 768 || (p->ny == 1024 && all) || p->M == 1 || (p->ny == 1024 && p->n_obs > 2) ||
+                (p->use_fused() && 2 * (p->L + 1) <= col_fused_groups(p->ny, 0));
+    if (work == kUpdateOnly) cols = split_update_columns(p);
+    // sums alone: 768x2048 N=3 4 blocks 122 -> 148, N=10 one of 3 observed 207 -> 234, 1024x2048 N=3 2 blocks 72 -> 84
+    else if (work == kEstimateOnly)
+      cols = cols && !(few_long && all && p->ny <= 1536 && (long long)p->ny * p->nx >= 1 << 20) &&
+             !(p->ny == 768 && p->nx >= 2048 && p->N < 16 && (all || p->n_obs == 1));
+    else if (p->ny == 1024 && all && p->n_obs > 1 && few_long) cols = false;
+    if (cols) bits |= kSplitCols;
   }
   if (p->L <= 1024 && (long long)p->M * p->N * p->ny * p->nx <= (1LL << 23)) bits |= kSplitInv;
   return bits;
@@ -453,7 +484,7 @@ extern "C" fftenkf_status fftenkf_estimate_spectrum(fftenkf_plan p, const void* 
   fftenkf_status st = get_workspace(p, workspace, &ws);
   if (st != FFTENKF_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int split = split_rule(p);
+  const int split = split_rule(p, kEstimateOnly);
   SplitParams q = split_params(p, ws, ensemble, nullptr, nullptr, nullptr);
   cudaError_t e = run_rows(p, q, true, 0, split, ws, s);
   if (split & kSplitCols) {
@@ -584,7 +615,7 @@ static fftenkf_status analyze_impl(fftenkf_plan p, void* ensemble, const float* 
   fftenkf_status st = get_workspace(p, workspace, &ws);
   if (st != FFTENKF_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int split = split_rule(p);
+  const int split = split_rule(p, spectrum ? kUpdateOnly : kEstimateAndUpdate);
   SplitParams q = split_params(p, ws, ensemble, data, perturbations, rhat);
   const int innovations = drawn ? kInnovationDrawn : kInnovation;
   cudaError_t e = cudaSuccess;

@@ -1,15 +1,27 @@
-"""The batched autotuner times the passes as real inputs run them: for a batch of one shape (its passes in series,
-in the tuner and in the replay) the tuned sum is the replay's time, within 20 % (three launches' gaps of a few us on
-about 0.5 ms, and the spread of runs).  With rhat = 0 in its scratch inputs every wavenumber took the columns' FP64
-branch and the sum came out far higher."""
+"""The batched autotuner times the passes as real inputs run them: its scratch rhat is a positive, ordinary double (with
+rhat = 0 every denominator vanishes, and every wavenumber takes a branch that real inputs do not); and for a batch of one shape
+(its passes in series, in the tuner and in the replay) the tuned sum is the replay's time, within 20 % (three launches'
+gaps of a few us on about 0.5 ms, and the spread of runs)."""
+
+import os
+import re
+import struct
 
 import pytest
 
 torch = pytest.importorskip("torch")
 
-pytestmark = pytest.mark.gpu
+SOURCE = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1001_1588_gb300", "csrc", "batch_api.cu")
 
 
+def test_scratch_rhat_is_an_ordinary_variance():
+    with open(SOURCE, encoding="utf-8") as f:
+        fill = re.search(r"cudaMemsetAsync\(scratch \+ field_bytes, (0x[0-9a-f]{2}), bytes - field_bytes, s\);", f.read())
+    rhat, = struct.unpack("<d", bytes([int(fill.group(1), 16)]) * 8)
+    assert 1e-6 < rhat < 1e3
+
+
+@pytest.mark.gpu
 def test_tuned_time_is_the_time_of_real_inputs():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")

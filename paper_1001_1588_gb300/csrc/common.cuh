@@ -239,6 +239,8 @@ struct SineParams {
   float inv_sqrt_N, scale, inv_G;   // scale = inv_G / (N-1), inv_G = 1 / (4 (ny-1)(nx-1))
   int* status;
 };
+// whether the sine passes' lines of P points read every twiddle power from their tables
+__host__ __device__ constexpr bool sine_every(int P) { return P % 3 != 0 && P <= 1024; }
 // threads of a column's CTA at most: 128 registers, or 255 with the coefficients of 3 or 4 observed blocks
 __host__ __device__ constexpr int sine_col_threads(int n_obs) { return n_obs <= 2 ? 512 : 256; }
 // thread groups of a column's CTA; 0 where the sine passes do not cover the shape

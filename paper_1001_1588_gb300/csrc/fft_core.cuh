@@ -314,44 +314,49 @@ template <bool INV> struct Dft<24, INV> : DftPrime3<8, INV> {};
 // radix-8 stages are one more rounding than a wide line's, and exact powers make up for it (relative RMS
 // error of 64 points 9.1e-8 with formed powers, 7.9e-8 with these, the wide plan 8.3e-8; 1024 points 12.0e-8,
 // 10.7e-8, 11.6e-8).
+// A caller may ask for every power (X) of another plan, with the table to match.
 __host__ __device__ constexpr bool tw_every(int N, int V) { return V == 8 && N <= 1024; }
-__host__ __device__ constexpr int tw_npow(int N, int V, int R) {
-  return tw_every(N, V) ? R - 1 : R > 16 ? 5 : R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : 1;
+__host__ __device__ constexpr int tw_npow(int R, bool X) {
+  return X ? R - 1 : R > 16 ? 5 : R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : 1;
 }
-__host__ __device__ constexpr int tw_pow(int N, int V, int q) { return tw_every(N, V) ? q + 1 : 1 << q; }   // the q-th stored power
+__host__ __device__ constexpr int tw_pow(int q, bool X) { return X ? q + 1 : 1 << q; }   // the q-th stored power
 __host__ __device__ constexpr int stage_ns(int N, int V, int s) {
   int ns = 1;
   for (int i = 0; i < s; ++i) ns *= radix_at(N, V, i);
   return ns;
 }
-__host__ __device__ constexpr int twiddle_offset(int N, int V, int s) {
+__host__ __device__ constexpr int twiddle_offset(int N, int V, int s, bool X) {
   int off = 0;
-  for (int i = 1; i < s; ++i) off += tw_npow(N, V, radix_at(N, V, i)) * stage_ns(N, V, i);
+  for (int i = 1; i < s; ++i) off += tw_npow(radix_at(N, V, i), X) * stage_ns(N, V, i);
   return off;
 }
-__host__ __device__ constexpr int twiddle_count(int N, int V) { return twiddle_offset(N, V, num_stages(N, V)); }
+__host__ __device__ constexpr int twiddle_count(int N, int V, bool X) { return twiddle_offset(N, V, num_stages(N, V), X); }
+__host__ __device__ constexpr int twiddle_count(int N, int V) { return twiddle_count(N, V, tw_every(N, V)); }
 // exponent e (of W_N^e = exp(-2 pi i e / N)) of table entry i, 0 <= i < twiddle_count(N, V)
-__host__ __device__ constexpr long long twiddle_exponent(int N, int V, int i) {
+__host__ __device__ constexpr long long twiddle_exponent(int N, int V, int i, bool X) {
   const int S = num_stages(N, V);
   int s = 1;
-  while (s + 1 < S && twiddle_offset(N, V, s + 1) <= i) ++s;
+  while (s + 1 < S && twiddle_offset(N, V, s + 1, X) <= i) ++s;
   const int NS = stage_ns(N, V, s), R = radix_at(N, V, s);
-  const int local = i - twiddle_offset(N, V, s);
+  const int local = i - twiddle_offset(N, V, s, X);
   const int q = local / NS, jm = local - q * NS;
-  return ((long long)jm * tw_pow(N, V, q) * (N / (NS * R))) % N;
+  return ((long long)jm * tw_pow(q, X) * (N / (NS * R))) % N;
+}
+__host__ __device__ constexpr long long twiddle_exponent(int N, int V, int i) {
+  return twiddle_exponent(N, V, i, tw_every(N, V));
 }
 
 // w^r for r = 1..R-1 of one butterfly from the stored powers (tws: this butterfly's
 // first entry; rows NS apart); conjugated for the inverse transform
-template <int N, int V, int R, bool INV>
+template <int R, bool INV, bool X>
 __device__ __forceinline__ void twiddle_powers(float2 (&w)[R], const float2* __restrict__ tws, int NS) {
 #pragma unroll
-  for (int q = 0; q < tw_npow(N, V, R); ++q) {
+  for (int q = 0; q < tw_npow(R, X); ++q) {
     float2 x = __ldg(tws + q * NS);
     if (INV) x.y = -x.y;
-    w[tw_pow(N, V, q)] = x;
+    w[tw_pow(q, X)] = x;
   }
-  if constexpr (tw_every(N, V)) return;
+  if constexpr (X) return;
 #pragma unroll
   for (int r = 3; r < R; ++r) {
     if ((r & (r - 1)) == 0) continue;          // stored
@@ -388,7 +393,7 @@ __device__ __forceinline__ int line_bar(int g) {
 // applies the R-point DFT and writes x[(j/NS) NS R + (j mod NS) + r NS].
 // Thread t owns butterflies j = t + T b (b < V/R), whose inputs are its
 // canonical slots b + r V/R; the last stage's outputs land in canonical slots.
-template <int N, int V, int S, int NS, bool INV, bool TRAIL>
+template <int N, int V, int S, int NS, bool INV, bool TRAIL, bool X>
 struct Stage {
   static __device__ __forceinline__ void run(float2 (&v)[V], float2* sm, int t, const float2* __restrict__ tw, int bid) {
     constexpr int R = radix_at(N, V, S);
@@ -403,7 +408,7 @@ struct Stage {
       const int j = t + T * b;
       if (NS > 1) {
         float2 w[R];
-        twiddle_powers<N, V, R, INV>(w, tw + twiddle_offset(N, V, S) + (j % NS), NS);
+        twiddle_powers<R, INV, X>(w, tw + twiddle_offset(N, V, S, X) + (j % NS), NS);
 #pragma unroll
         for (int r = 1; r < R; ++r) a[r] = cmul(a[r], w[r]);
       }
@@ -424,7 +429,7 @@ struct Stage {
       // the buffer is written again by the next stage, or (after the last exchange) by the caller;
       // without TRAIL the caller synchronises before it reuses the buffer
       if constexpr (TRAIL || S + 2 < num_stages(N, V)) line_sync<T>(bid);
-      Stage<N, V, S + 1, NS * R, INV, TRAIL>::run(v, sm, t, tw, bid);
+      Stage<N, V, S + 1, NS * R, INV, TRAIL, X>::run(v, sm, t, tw, bid);
     }
   }
 };
@@ -434,13 +439,13 @@ struct Stage {
 // with line_sync(bid) when the plan has >1 stage.  With TRAIL = false it returns
 // while other threads of the line may still read sm: the caller must pass a
 // barrier of those threads before anything writes sm again.
-// tw: the stage-major twiddle table of (N, V) described above (exp(-2 pi i e/N)
+// tw: the stage-major twiddle table of (N, V, X) described above (exp(-2 pi i e/N)
 // values).  sm: this line's padded buffer.
-template <int N, int V, bool INV, bool TRAIL = true>
+template <int N, int V, bool INV, bool TRAIL = true, bool X = tw_every(N, V)>
 __device__ __forceinline__ void fft_line(float2 (&v)[V], float2* sm, int t, const float2* __restrict__ tw, int bid = 0) {
   static_assert(N % V == 0, "V must divide N");
   static_assert(num_stages(N, V) > 0, "no radix plan");
-  Stage<N, V, 0, 1, INV, TRAIL>::run(v, sm, t, tw, bid);
+  Stage<N, V, 0, 1, INV, TRAIL, X>::run(v, sm, t, tw, bid);
 }
 
 }  // namespace fftenkf

@@ -141,7 +141,7 @@ struct PStage {
       const int j = t + T * b;
       if (NS > 1) {
         float2 w[R];
-        twiddle_powers<N, V, R, INV>(w, tw + twiddle_offset(N, V, S) + (j % NS), NS);
+        twiddle_powers<R, INV, tw_every(N, V)>(w, tw + twiddle_offset(N, V, S, tw_every(N, V)) + (j % NS), NS);
 #pragma unroll
         for (int r = 1; r < R; ++r) a[r] = cp_mulw(a[r], w[r]);
       }
@@ -188,7 +188,7 @@ struct PStage2 {
       const int j = t + T * b;
       if (NS > 1) {
         float2 w[R];
-        twiddle_powers<N, V, R, INV>(w, tw + twiddle_offset(N, V, S) + (j % NS), NS);
+        twiddle_powers<R, INV, tw_every(N, V)>(w, tw + twiddle_offset(N, V, S, tw_every(N, V)) + (j % NS), NS);
 #pragma unroll
         for (int r = 1; r < R; ++r) a[r] = cp_mulw(a[r], w[r]);
       }

@@ -24,6 +24,15 @@ namespace fftenkf {
 // tiles of 4 would take 916 us instead of 870)
 __host__ __device__ constexpr int sine_tile_lines(int P) { return P >= 4096 ? 2 : 4; }
 
+// The line transforms of the sine passes; power-of-two lines up to 1024 points with every twiddle power from the
+// table: they are twice as long as the periodic passes' rows of the same grid, and with formed powers FP32 analyses
+// were further from the 64-bit result than through the extension (65^2 nodes, N=5, 2 blocks 3.1e-7 and 2.8e-7, mean
+// of three draws; 2.5e-7 like this, at the same speed: 1025^2 1543 us both).
+template <int P, int V, bool TRAIL = true>
+__device__ __forceinline__ void sine_line(float2 (&v)[V], float2* line, int t, const float2* __restrict__ tw, int bid) {
+  fft_line<P, V, false, TRAIL, sine_every(P)>(v, line, t, tw, bid);
+}
+
 template <int ST>
 __device__ __forceinline__ float load1(const void* base, size_t idx) {
   if constexpr (ST == kBF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(base)[idx]);
@@ -127,7 +136,7 @@ __global__ void __launch_bounds__(256, 2) sine_rows_kernel(const __grid_constant
     }
     float2* line = lines + (l + g) * pitch;
     odd_extension<P, V>(v, line, t, line_bar<T>(g));
-    fft_line<P, V, false>(v, line, t, p.twx, line_bar<T>(g));
+    sine_line<P, V>(v, line, t, p.twx, line_bar<T>(g));
     float* fa = reinterpret_cast<float*>(line);   // T(a) = -Im Z, T(b) = Re Z at k = 0..n-1
 #pragma unroll
     for (int m = 0; m < V / 2; ++m) {
@@ -188,7 +197,7 @@ __global__ void __launch_bounds__(256, 2) sine_rows_inv_kernel(const __grid_cons
 #pragma unroll
     for (int m = 0; m < V; ++m) v[m] = line[pidx(t + T * m)];
     line_sync<T>(line_bar<T>(g));
-    fft_line<P, V, false, false>(v, line, t, p.twx, line_bar<T>(g));
+    sine_line<P, V, false>(v, line, t, p.twx, line_bar<T>(g));
 #pragma unroll
     for (int m = 0; m < V / 2; ++m) {
       const int x = t + T * m;
@@ -240,7 +249,7 @@ __global__ void __launch_bounds__(sine_col_threads(NOBS), 1) sine_cols_kernel(co
       v[m] = make_float2(in ? f[col + y - 1] : 0.f, in && two ? f[col + n + y - 1] : 0.f);
     }
     odd_extension<P, V>(v, line, t, bid);
-    fft_line<P, V, false>(v, line, t, p.twy, bid);
+    sine_line<P, V>(v, line, t, p.twy, bid);
 #pragma unroll
     for (int m = 0; m < H; ++m) {
       c[m] = -v[m].y;
@@ -345,7 +354,7 @@ __global__ void __launch_bounds__(sine_col_threads(NOBS), 1) sine_cols_kernel(co
         v[m] = make_float2(in ? s[m] : 0.f, in && two ? s[H + m] : 0.f);
       }
       odd_extension<P, V>(v, line, t, bid);
-      fft_line<P, V, false>(v, line, t, p.twy, bid);
+      sine_line<P, V>(v, line, t, p.twy, bid);
       if (!act) continue;
       float* o = p.A + ((size_t)p.role_block[r] * N + k) * p.fstride + col;
 #pragma unroll

@@ -231,8 +231,8 @@ static cudaError_t native_setup(fftenkf_sine_plan_s* p, const uint8_t* observed_
   for (int d = 0; d < 2; ++d) {
     off[d] = tw.size();
     const int V = plan_V(len[d], 0);
-    for (int i = 0; i < twiddle_count(len[d], V); ++i) {
-      const double ang = 2.0 * M_PI * (double)twiddle_exponent(len[d], V, i) / (double)len[d];
+    for (int i = 0; i < twiddle_count(len[d], V, sine_every(len[d])); ++i) {
+      const double ang = 2.0 * M_PI * (double)twiddle_exponent(len[d], V, i, sine_every(len[d])) / (double)len[d];
       tw.push_back(make_float2((float)std::cos(ang), (float)-std::sin(ang)));
     }
     tw.push_back(make_float2(0.f, 0.f));

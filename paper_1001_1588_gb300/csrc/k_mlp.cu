@@ -396,23 +396,59 @@ __device__ __forceinline__ void mlp_delta(const float* W, const float* d, const 
   __syncthreads();
 }
 
+// Back-propagation of the CTA's samples from the output deltas in d0
+template <int S>
+__device__ __forceinline__ void mlp_gradients(const MlpGradParams& p, const MlpActs<S>& a, float* d0, float* d1, float* part,
+                                              bool gvec, int tid) {
+  mlp_weight_grads<S, kH, kOut>(p.grads + kOffW4, p.grads + kOffB4, gvec, d0, &a.h[2][0][0], tid);
+  mlp_delta<S, kOut>(p.params + kOffW4, d0, &a.z[2][0][0], part, d1, tid);
+  mlp_weight_grads<S, kH, kH>(p.grads + kOffW3, p.grads + kOffB3, gvec, d1, &a.h[1][0][0], tid);
+  mlp_delta<S, kH>(p.params + kOffW3, d1, &a.z[1][0][0], part, d0, tid);
+  mlp_weight_grads<S, kH, kH>(p.grads + kOffW2, p.grads + kOffB2, gvec, d0, &a.h[0][0][0], tid);
+  mlp_delta<S, kH>(p.params + kOffW2, d0, &a.z[0][0][0], part, d1, tid);
+  mlp_weight_grads<S, kIn, kH>(p.grads + kOffW1, p.grads + kOffB1, gvec, d1, &a.x[0][0], tid);
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// *x of the cluster's first CTA = v
+__device__ __forceinline__ void store_to_first(float* x, float v) {
+  uint32_t at;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(x)));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(at), "f"(v) : "memory");
+}
+
 // Gradient of mean((out - target)^2) over all B x 128 outputs: forward pass of S samples per CTA, then
 // back-propagation; grads and loss zeroed before.  At this size the work is a chain of short phases, so
 // what counts is latency and conflict-free operand access: batch 256 took 60 us with the weights staged in shared
 // memory (32-way bank conflicts of the row-major weights), 8 samples per CTA and scalar atomics; a gradient
-// and Adam step of that batch went from 71.9 to 26.9 us.
+// and Adam step of that batch went from 71.9 to 29.2 us (26.9 without the pairs below).
+//
+// The losses of the CTAs are added in FP32 in free order, with an error that grows with their number.  CTAs of four
+// samples come in clusters of two, which add their losses first (through the pair's distributed shared memory), so
+// that as many terms are added as with eight samples per CTA.  (Relative error against 64 bits, root mean square over
+// 24 batches: of 600 samples 2.1e-7 without, 1.5e-7 like this, 1.2e-7 the first kernel above; of 256 1.0e-7, 0.6e-7 and
+// 0.8e-7.  The gradients of 256 are 1.7e-7 off, 1.5e-7 with eight samples per CTA, 2.8e-7 with the first kernel.)
 template <int S>
 __global__ void __launch_bounds__(256) mlp_bwd_kernel(const MlpGradParams p) {
+  constexpr bool PAIR = S == 4;   // launched in clusters of two
   __shared__ MlpActs<S> a;
   __shared__ alignas(16) float d0[kOut * S];
   __shared__ alignas(16) float d1[kH * S];
   __shared__ float part[4 * kH * S];
   __shared__ float red8[8];
-  const int s0 = blockIdx.x * S, nsamp = min(S, p.B - s0), tid = threadIdx.x;
+  __shared__ float partner;   // the second CTA's loss, in the first
+  const int s0 = blockIdx.x * S, nsamp = min(S, p.B - s0), tid = threadIdx.x;   // nsamp <= 0: completes a pair
   const bool vec = (reinterpret_cast<uintptr_t>(p.params) & 15) == 0;
   const bool gvec = (reinterpret_cast<uintptr_t>(p.grads) & 15) == 0;
   stream_order_wait();
   next_may_start();
+  if constexpr (PAIR) cluster_arrive();
   load_samples<S>(a, p.X, s0, nsamp, 256);
   mlp_forward<S, 8>(a, p.params, vec, tid >> 5, tid & 31);
   const float scale = 2.f / ((float)p.B * kOut);
@@ -424,14 +460,18 @@ __global__ void __launch_bounds__(256) mlp_bwd_kernel(const MlpGradParams p) {
     d0[o * S + s] = scale * diff;
   }
   const float t = block_sum256(l, red8);   // holds a barrier: d0 is complete after it
-  if (tid == 0) atomicAdd(p.loss, t / ((float)p.B * kOut));
-  mlp_weight_grads<S, kH, kOut>(p.grads + kOffW4, p.grads + kOffB4, gvec, d0, &a.h[2][0][0], tid);
-  mlp_delta<S, kOut>(p.params + kOffW4, d0, &a.z[2][0][0], part, d1, tid);
-  mlp_weight_grads<S, kH, kH>(p.grads + kOffW3, p.grads + kOffB3, gvec, d1, &a.h[1][0][0], tid);
-  mlp_delta<S, kH>(p.params + kOffW3, d1, &a.z[1][0][0], part, d0, tid);
-  mlp_weight_grads<S, kH, kH>(p.grads + kOffW2, p.grads + kOffB2, gvec, d0, &a.h[0][0][0], tid);
-  mlp_delta<S, kH>(p.params + kOffW2, d0, &a.z[0][0][0], part, d1, tid);
-  mlp_weight_grads<S, kIn, kH>(p.grads + kOffW1, p.grads + kOffB1, gvec, d1, &a.x[0][0], tid);
+  if constexpr (PAIR) {
+    cluster_wait();   // both CTAs have started
+    if (tid == 0 && cluster_rank() == 1) store_to_first(&partner, t);
+    cluster_arrive();
+  } else {
+    if (tid == 0) atomicAdd(p.loss, t / ((float)p.B * kOut));
+  }
+  if (nsamp > 0) mlp_gradients<S>(p, a, d0, d1, part, gvec, tid);
+  if constexpr (PAIR) {
+    cluster_wait();   // the partner's loss has arrived
+    if (tid == 0 && cluster_rank() == 0) atomicAdd(p.loss, (t + partner) / ((float)p.B * kOut));
+  }
 }
 
 struct MlpAdamParams {
@@ -523,20 +563,19 @@ cudaError_t launch_mlp_denoise(const double* chat_in, const MlpBins& t, const fl
 
 cudaError_t launch_mlp_forward(const float* params, const float* X, int B, float* out, cudaStream_t s) {
   const MlpFwdParams p{params, X, out, B};
+  // a sample per CTA of 32 warps up to two such CTAs per SM (batch 304: 8.0 us, 20.7 with eight samples per CTA)
   if (B <= 304) return launch_overlapped(mlp_fwd_kernel<1, 32>, dim3(B), 1024, 0, s, p);
   return launch_overlapped(mlp_fwd_kernel<8, 8>, dim3((B + 7) / 8), 256, 0, s, p);
 }
 
-// 4 samples per CTA up to 16 CTAs, then 8: the gradient's error grows with the number of partial sums that are added
-// in free order (batch 256: relative error against 64 bits 1.43e-7 with 8 samples per CTA, 1.68e-7 with 4; 608:
-// 1.63e-7 and 2.03e-7; 64: 1.76e-7 and 1.79e-7).  4 samples are faster up to one CTA per SM (batch 256: 24.1 us
-// against 27.8).
+// 4 samples per CTA, in pairs, up to one CTA per SM of a 152-SM GPU (with Adam, batch 256: 29.2 us, 31.4 with 8), then
+// 8 (half the atomics)
 cudaError_t launch_mlp_gradient(const float* params, const float* X, const float* target, int B, float* grads,
                                 float* loss, cudaStream_t s) {
   const MlpGradParams p{params, X, target, grads, loss, B};
   cudaError_t e = launch_overlapped(mlp_zero_kernel, dim3((kParams + 255) / 256), 256, 0, s, p);
   if (e != cudaSuccess) return e;
-  if (B <= 64) return launch_overlapped(mlp_bwd_kernel<4>, dim3((B + 3) / 4), 256, 0, s, p);
+  if (B <= 608) return launch_overlapped(mlp_bwd_kernel<4>, dim3(2 * ((B + 7) / 8)), 256, 0, s, p, 2);
   return launch_overlapped(mlp_bwd_kernel<8>, dim3((B + 7) / 8), 256, 0, s, p);
 }
 

@@ -24,21 +24,24 @@ __device__ __forceinline__ void stream_order_wait() { asm volatile("griddepcontr
 // 4 blocks 346 and 259; 64^2 14 us both; called before a CTA's last stores: 35, 270, 14).
 __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Launch with the stream's order kept by stream_order_wait() at the kernel's start: the launch latency
+// Launch (of clusters of `cluster` CTAs) with the stream's order kept by stream_order_wait() at the kernel's start: the launch latency
 // of a kernel overlaps the one before it (2-3 us between dependent kernels otherwise).
 template <typename P>
 inline cudaError_t launch_overlapped(void (*kern)(const P), dim3 grid, int threads, size_t smem, cudaStream_t st,
-                                     const P& p) {
+                                     const P& p, unsigned cluster = 1) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, p);
 }
 

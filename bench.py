@@ -815,7 +815,7 @@ def run_ours(a):
         out = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
             "warmup": a.warmup, "ms_per_step": step_ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "f32 (bf16 storage, f64 gain)", "data": "synthetic",
+            "vs_baseline": None, "dtype": "f32 (bf16 storage, gains beyond f32)", "data": "synthetic",
             "config": {"workload": WORKLOAD, "grid": [ny, nx], "members": Nm, "blocks": M, "observed": N_OBS,
                        "l2": "inputs larger than L2 (2.7 GB ensemble re-read every step)",
                        "parallelism": "independent analysis per GPU" if world > 1 else "single GPU"},

@@ -6,11 +6,10 @@
 // pass over the units of its items: forward rows (anomalies and innovations), columns, inverse rows.  The
 // kernels take the pointers of an item from a device table, so that new pointers need a new table and no
 // new graph.  The classes are issued on kLanes graph branches, largest first, each to the branch with the
-// least work (cut into chunks of 48 to 160 MB, whose spectra stay in L2, the batch below takes 8.6 to 10.4 ms
-// instead of 8.07).  (256 mixed analyses, 8 to
-// 1024 points a side, FP32: 12.32 -> 8.16 ms.  Before, the 103 analyses of at least 512 x 256 points ran on
-// plans of their own, whose kernels each filled a fraction of the SMs, and the others in seven persistent
-// launches whose units were serial over the members.)
+// least work.  256 mixed analyses, 32 to 1024 points a side, FP32: 7.9 ms; 12.32 with the 103 analyses of
+// at least 512 x 256 points on plans of their own, whose kernels each filled a fraction of the SMs, and the others in
+// seven persistent launches whose units were serial over the members; 8.6 to 10.4 (then 8.07) cut into chunks of
+// 48 to 160 MB, whose spectra stay in L2.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

@@ -185,9 +185,9 @@ struct SplitParams {
   int anomalies;          // forward rows: the anomalies are transformed
   int innovations;        // forward rows: 0, kInnovation or kInnovationDrawn
   const float2 *twL, *twX, *twY;   // tables of split_row_V(L), plan_V(ny, split_col_sel)
-  int R;                  // rows per tile (set by split_row_shape)
+  int R;                  // rows per tile (set by launch_rows_split)
   int threads;            // batched: threads of a CTA (0 = default)
-  int groups;             // thread groups of the column pass (set by split_col_shape)
+  int groups;             // thread groups of the column pass (set by launch_col_split; batched: by the caller)
   int acc_bytes;          // shared memory of its sums
   float* chat;            // columns: covariance tables wanted instead of the update, in the col_stats layout
   const double* spec;     // columns: caller's spectrum tables in place of the sums
@@ -202,7 +202,11 @@ __host__ __device__ constexpr int split_row_V(int L) {
   return L % 3 == 0 ? (L >= 192 ? 24 : (L >= 12 ? 12 : L)) : (L >= 128 ? 16 : (L >= 8 ? 8 : L));
 }
 // line plan (plan_V selector) of the split columns: wide lines without cross sums, whose threads keep the
-// sums in registers; narrow ones for short lines and with cross sums
+// sums in registers; narrow ones for short lines and with cross sums.  512 points are near the line (columns of
+// 512 x 512 N=20 28.1 us narrow, 28.8 wide, of two observed blocks 51.0 and 55.2, 512 x 1024 BF16 N=20 49.5 and
+// 53.1, but 512 x 2048 BF16 N=10 57.2 and 51.5).  The wide plans of 192 points on spill for 3*2^a lines (470 to 680
+// bytes a thread with one observed block, 1.3 to 1.7 KB with two, over 4 with three or four); where that costs more than the pipelined
+// passes, split_rule (api.cu) knows.
 __host__ __device__ constexpr int split_col_sel(int ny, bool cross) {
   return (cross || (ny % 3 == 0 ? ny < 192 : (ny < 128 || ny == 512))) ? 1 : 0;
 }

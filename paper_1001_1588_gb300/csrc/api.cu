@@ -290,11 +290,12 @@ static fftenkf_status get_workspace(fftenkf_plan p, void* ws, char** out) {
 //     the SMs (256x4096 N=4 66 -> 39, but 512x4096 N=20 4 blocks 597 -> 841); FP32 rows of 384 points (24 values on
 //     each of 8 threads) not with many members on long columns (estimate of 1536x384 N=25 3 blocks 343 -> 415,
 //     3072x384 615 -> 692; but 2048x384 536 -> 498, and BF16 of 1536x384 551 -> 371)
-//   columns: up to 768 points always (512^2 N=5 3 blocks 101 -> 30, 512x4096 N=20 4 blocks 683 -> 598); above, with one observed and no other block (1024^2 N=20 163 -> 100, 2048^2
-//     N=10 352 -> 213), with all blocks observed at 1024 (186 -> 187, two launches fewer; but not for few members
-//     on long rows, 1024x2048 N=3 4 blocks 438 -> 517, 1024x4096 N=3 2 blocks 348 -> 387), where the fused pass does
-//     not apply for the observed blocks (1024x2048 N=15, 3 of 4 observed 851 -> 672), and where the fused pass would
-//     leave more than half its column groups idle (1024x512 N=8 167 -> 104, but 1024^2 N=20 192 -> 218)
+//   columns: up to 768 points always (512^2 N=5 3 blocks 101 -> 30, 512x4096 N=20 4 blocks 683 -> 598); above, with
+//     one observed and no other block (1024^2 N=20 163 -> 100, 2048^2 N=10 352 -> 213), with all blocks observed at
+//     1024 (186 -> 187, two launches fewer; but not for few members on long rows, 1024x2048 N=3 4 blocks 438 -> 517,
+//     1024x4096 N=3 2 blocks 348 -> 387), where the fused pass does not apply for the observed blocks (1024x2048 N=15,
+//     3 of 4 observed 851 -> 672), and where it would leave more than half its column groups idle (1024x512 N=8
+//     167 -> 104, but 1024^2 N=20 192 -> 218)
 //   inverse rows: up to 2^23 points of the ensemble and 2048-point rows (1024^2 N=5 25 -> 21, but N=20 65 -> 72)
 enum SplitBits { kSplitRows = 1, kSplitCols = 2, kSplitInv = 4 };
 // what a call's columns do: sums, gains and update; the sums alone; the update with gains of a caller's spectrum

@@ -205,8 +205,8 @@ __host__ __device__ constexpr int split_row_V(int L) {
 // sums in registers; narrow ones for short lines and with cross sums.  512 points are near the line (columns of
 // 512 x 512 N=20 28.1 us narrow, 28.8 wide, of two observed blocks 51.0 and 55.2, 512 x 1024 BF16 N=20 49.5 and
 // 53.1, but 512 x 2048 BF16 N=10 57.2 and 51.5).  The wide plans of 192 points on spill for 3*2^a lines (470 to 680
-// bytes a thread with one observed block, 1.3 to 1.7 KB with two, over 4 with three or four); where that costs more than the pipelined
-// passes, split_rule (api.cu) knows.
+// bytes a thread with one observed block, 1.3 to 1.7 KB with two, over 4 with three or four); split_rule (api.cu)
+// takes the pipelined passes where that costs more than them.
 __host__ __device__ constexpr int split_col_sel(int ny, bool cross) {
   return (cross || (ny % 3 == 0 ? ny < 192 : (ny < 128 || ny == 512))) ? 1 : 0;
 }
